@@ -48,6 +48,7 @@ struct cc_graph {
   uint32_t push_cap = 0;
   uint32_t *cand_list = nullptr;  // listed candidates of the root selection (cand_cap entries), f = R only
   uint32_t cand_cap = 0;
+  cc::WideHot *wide_hot = nullptr;  // wide hot-vertex table, or null
   uint32_t *z = nullptr;   // zero-tree bitmap (one bit per name), or null
   size_t z_bytes = 0;
   bool z_forced = false;   // CC_FILTER_BITMAP: always used
@@ -76,6 +77,14 @@ uint32_t push_cap_for(uint64_t n) {
 bool wants_z(const cc_options &o, uint64_t n) {
   if (o.filter == CC_FILTER_BITMAP) return true;
   return o.filter == CC_FILTER_AUTO && o.mode == CC_ROOT_MAXDEG && (uint64_t)n * 4 >= kZMinBytes;
+}
+
+// The wide hot-vertex table: exact selection (it is filled from its sample) and
+// the edge pass's default shape.
+bool wants_wide_hot(const cc_options &o, uint64_t n) {
+  return o.mode == CC_ROOT_MAXDEG && o.root_hint == CC_ROOT_AUTO && o.root_select != CC_ROOT_SELECT_SAMPLED &&
+         o.filter != CC_FILTER_OFF && o.filter != CC_FILTER_BITMAP && o.block_size == 0 && o.edges_per_thread == 0 &&
+         cc::wide_hot_fits(n);
 }
 
 struct DeviceGuard {
@@ -199,7 +208,7 @@ cc_status root_select(cc_graph *g, const uint32_t *edges, uint64_t n_edges, cons
     return CC_OK;
   }
   CC_TRY(cc::launch_root_select_certified(edges, n_edges, span, g->cnt, wide, n, g->cert, g->ctrl, s, g->push,
-                                         g->push_cap, g->cand_list, g->cand_cap));
+                                         g->push_cap, g->cand_list, g->cand_cap, g->wide_hot));
   return CC_OK;
 }
 
@@ -282,7 +291,7 @@ cc_status cc_create(uint64_t n_vertices, uint64_t n_edges_capacity, const cc_opt
   const bool rf = o.mode == CC_ROOT_MAXDEG;
   const size_t need = p_bytes(n_vertices) +
                       (rf ? (size_t)n_vertices * 4 + sizeof(cc::CertScratch) + (size_t)cc::cand_list_cap(n_vertices) * 4
-                          : 0) + sizeof(Ctrl) +
+                          : 0) + sizeof(Ctrl) + (wants_wide_hot(o, n_vertices) ? sizeof(cc::WideHot) : 0) +
                       (size_t)n_edges_capacity * 8 + (wants_z(o, n_vertices) ? z_bytes_for(n_vertices) : 0) +
                       (wants_push(o) ? (size_t)push_cap_for(n_vertices) * 4 : 0);
   if (o.hbm_budget_bytes && need > o.hbm_budget_bytes) return CC_ERR_OOM;
@@ -315,6 +324,9 @@ cc_status cc_create(uint64_t n_vertices, uint64_t n_edges_capacity, const cc_opt
       if ((e = dev_alloc(g, (void **)&g->cert, sizeof(cc::CertScratch))) != cudaSuccess) break;
       g->cand_cap = cc::cand_list_cap(n_vertices);
       if ((e = dev_alloc(g, (void **)&g->cand_list, (size_t)g->cand_cap * 4)) != cudaSuccess) break;
+      if (wants_wide_hot(o, n_vertices) &&
+          (e = dev_alloc(g, (void **)&g->wide_hot, sizeof(cc::WideHot))) != cudaSuccess)
+        break;
     }
     if (n_edges_capacity) {
       if ((e = dev_alloc(g, (void **)&g->staging, (size_t)n_edges_capacity * 8)) != cudaSuccess) break;
@@ -359,6 +371,7 @@ void cc_destroy(cc_graph *g) {
   dev_free(g, g->cnt, g->cnt_bytes);
   dev_free(g, g->cert, sizeof(cc::CertScratch));
   dev_free(g, g->cand_list, (size_t)g->cand_cap * 4);
+  dev_free(g, g->wide_hot, sizeof(cc::WideHot));
   dev_free(g, g->ctrl, sizeof(Ctrl));
   dev_free(g, g->staging, (size_t)g->capacity * 8);
   dev_free(g, g->label_dev, (size_t)g->n * 4);
@@ -414,7 +427,7 @@ cc_status cc_run(cc_graph *g, const uint32_t *edges_dev, uint64_t n_edges, uint3
   record(g, 2, s);
   CC_TRY(cc::launch_edge_pass(g->rf, eff_filter(g), eff_ept(g), eff_block(g), span, g->P, n, g->ctrl,
                               nullptr, s, Z, zsel, false, nullptr, exact ? &g->ctrl->cert : nullptr, true,
-                              exact ? g->cert->hot : nullptr));
+                              exact ? g->cert->hot : nullptr, exact ? g->wide_hot : nullptr));
   record(g, 3, s);
   CC_TRY(cc::launch_flatten(g->rf, g->opt.label_space, g->P, n, L_out_dev, g->ctrl, s));
   record(g, 4, s);

@@ -65,6 +65,16 @@ __device__ __forceinline__ uint4 ld_edges(const uint4 *a, uint64_t pol) {
   return r;
 }
 
+// The same, kept where it stands in the program: for loads issued ahead of
+// their use, which the compiler would move down to it.
+__device__ __forceinline__ uint4 ld_edges_now(const uint4 *a, uint64_t pol) {
+  uint4 r;
+  asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v4.u32 {%0,%1,%2,%3}, [%4], %5;"
+               : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
+               : "l"(a), "l"(pol));
+  return r;
+}
+
 __device__ __forceinline__ uint2 ld_edge(const uint2 *a) {
   uint2 r;
   asm("ld.global.nc.L1::no_allocate.v2.u32 {%0,%1}, [%2];" : "=r"(r.x), "=r"(r.y) : "l"(a));
@@ -263,6 +273,15 @@ __device__ __forceinline__ void zset(uint32_t *Z, uint32_t c) {
 // Slot of vertex x in the hot-vertex table (kHot entries).
 __device__ __forceinline__ uint32_t hot_slot(uint32_t x) { return (x * 2654435761u) >> (32 - kHotBits); }
 
+// The wide table's bijection: mix, then bucket from the top bits of the s-bit
+// product; the low s - kWideBits bits tell the bucket's vertices apart.
+constexpr uint32_t kWideMul = 2654435761u, kWideInv = 244002641u;  // inverse of each other modulo 2^32
+static_assert(kWideMul * kWideInv == 1u, "the mix is undone by the inverse");
+__device__ __forceinline__ uint32_t wide_mix(uint32_t x) { return x * kWideMul; }
+__device__ __forceinline__ uint32_t wide_bucket(uint32_t y, uint32_t s_bits) {
+  return (y << (32u - s_bits)) >> (32u - kWideBits);
+}
+
 // A changed-root log: log[0] counts the entries that follow it, the names of
 // the roots hooked since the log was last cleared. Its capacity (one entry
 // per vertex) cannot be exceeded: a root is hooked once.
@@ -309,6 +328,7 @@ struct WarpRing {
   __device__ __forceinline__ void push(uint32_t *S, bool keep, uint32_t a, uint32_t pa, uint32_t b,
                                        uint32_t pb) {
     const uint32_t bal = __ballot_sync(0xFFFFFFFFu, keep);
+    if (!bal) return;
     // one call of unite() serves both routes: a second inlined copy cost
     // the plain pass a register spill
     const bool direct = (uint32_t)__popc(bal) >= direct_min;  // warp-uniform

@@ -162,6 +162,35 @@ struct CertScratch {
 };
 constexpr uint32_t kPushLanes = 256;
 
+// The wide hot-vertex table of the edge pass on large graphs (wide_hot_fits):
+// kWideBuckets words of up to kWideMaxWays fields. A vertex of a graph on at
+// most 2^s vertices is mixed by a bijection of [0, 2^s) (an odd multiplier)
+// whose top kWideBits bits name the bucket, so the other s - kWideBits bits
+// tell the vertices of a bucket apart exactly; a field holds them and a flag.
+// Filled by the candidate scan from the sampled counts, the largest counts of
+// a bucket first; the sampled pass then lists vertices from kWideListThr
+// occurrences up (edge pass of R-MAT scale 24 with thresholds 2, 3, 4 and 6:
+// 1.73, 1.74, 1.75, 1.80 ms in a first form of the pass).
+constexpr uint32_t kWideBits = 15;
+constexpr uint32_t kWideBuckets = 1u << kWideBits;
+constexpr uint32_t kWideMaxWays = 4;
+constexpr uint32_t kWideListThr = 3;
+struct WideHot {
+  uint32_t word[kWideBuckets];                          // the packed fields, flags clear
+  unsigned long long slot[kWideMaxWays][kWideBuckets];  // (sampled count << 32) | (vertex + 1), best first
+};
+// Smallest s with n <= 2^s.
+inline uint32_t id_bits(uint64_t n) {
+  uint32_t s = 0;
+  while ((1ULL << s) < n) ++s;
+  return s;
+}
+inline bool wide_hot_fits(uint64_t n) { return n >= (1ULL << 22) && n <= (1ULL << 30); }
+inline uint32_t wide_ways(uint32_t s) {
+  const uint32_t w = 32u / (s - kWideBits + 1u);
+  return w < kWideMaxWays ? w : kWideMaxWays;
+}
+
 // Chunked exact root selection, for edges that arrive in chunks (host input):
 // a dense sample of the first chunk picks candidates, and every chunk is
 // hooked under a speculative m' as it lands. With a plausible hub, m' is the
@@ -195,11 +224,12 @@ cudaError_t chunked_select_end(const EdgeSpan &all, void *cnt, bool wide, uint32
 // receives the neighbours of the sampled argmax during the counting pass, for
 // launch_initial_push after init. list (list_cap entries), when not null,
 // receives the listed candidates (kListThr) and the candidate scan reads it
-// instead of the n counters.
+// instead of the n counters. wide_hot, when not null (with a list), receives
+// the wide hot-vertex table.
 cudaError_t launch_root_select_certified(const uint32_t *edges, uint64_t n_edges, const EdgeSpan &e,
                                          void *cnt, bool wide, uint32_t n, CertScratch *cs, Ctrl *ctrl,
                                          cudaStream_t s, uint32_t *push_buf = nullptr, uint32_t push_cap = 0,
-                                         uint32_t *list = nullptr, uint32_t list_cap = 0);
+                                         uint32_t *list = nullptr, uint32_t list_cap = 0, WideHot *wide_hot = nullptr);
 // Initial Push (Algorithm 4): right after init, when the planted m is the
 // vertex whose neighbours were gathered, every gathered neighbour x != m gets
 // P[x] = 0 (name 0 is m): x, still a root, is hooked under m.
@@ -224,7 +254,8 @@ cudaError_t launch_unpack3(const uint8_t *src, uint64_t n_edges, uint32_t *dst, 
 cudaError_t launch_degree_sampled_u32(const uint2 *edges, uint64_t n_edges, uint64_t edge_base,
                                       uint32_t stride, uint32_t *cnt, uint32_t n, cudaStream_t s,
                                       Ctrl *track = nullptr, uint32_t *list = nullptr,
-                                      unsigned int *list_n = nullptr, uint32_t list_cap = 0);
+                                      unsigned int *list_n = nullptr, uint32_t list_cap = 0,
+                                      uint32_t list_thr = kListThr);
 cudaError_t launch_argmax_u32(const uint32_t *cnt, uint32_t n, Ctrl *ctrl, cudaStream_t s);
 // Z: the zero-tree bitmap (one bit per name, zeroed at every init), or null.
 // With Z and zsel null only the zero-tree instance runs; with both, the device
@@ -234,12 +265,13 @@ cudaError_t launch_argmax_u32(const uint32_t *cnt, uint32_t n, Ctrl *ctrl, cudaS
 // log: a changed-root log (log[0] = entries, then the hooked root names), or
 // null.
 // hot: the hot-vertex table (CertScratch::hot) of this graph's last root
-// selection, for the instances that serve a certified hub, or null.
+// selection, for the instances that serve a certified hub, or null; wide_hot:
+// the wide table, which takes its place on the default launch shape.
 cudaError_t launch_edge_pass(bool rf, int filter, int ept, int block, const EdgeSpan &e, uint32_t *P,
                              uint32_t n, Ctrl *ctrl, const uint32_t *skip, cudaStream_t s,
                              uint32_t *Z = nullptr, const uint32_t *zsel = nullptr, bool one_shot = false,
                              uint32_t *log = nullptr, const uint32_t *hub = nullptr, bool dyn = false,
-                             const unsigned long long *hot = nullptr);
+                             const unsigned long long *hot = nullptr, const WideHot *wide_hot = nullptr);
 // dyn: warps claim their edges from a counter in ctrl (reset on s before the
 // launch), so at most one dynamic edge pass per Ctrl may be in flight.
 // Sets *reject (ctrl->reject when null) and the range error bit when an id is >= n.

@@ -310,6 +310,205 @@ __global__ void __launch_bounds__(512, Q >= 4 ? (kZ ? 1 : 2) : (kZ ? 2 : (kDirec
   ring.drain<kCG>(S);
 }
 
+// The edge pass of a certified hub on a large graph (from 2^22 vertices up,
+// default launch shape): as the hub forms above, with the wide hot-vertex
+// table (WideHot) in place of the 4096-entry one.
+//
+// What bounds it: the endpoint lookups, one L2 request each, at most 0.96 per
+// SM and clock; random shared-memory loads beside them cost nothing (16 per 8
+// lookups left the rate at 0.96). So one block of 1024 threads per SM gives
+// 128 KB of its shared memory to the table, which answers 32 warps' lookups
+// of the hottest vertices: on R-MAT scale 24 (98K entries) L2 requests fell
+// from 489M to 348M. Edge pass before and after: R-MAT scale 28 31.24 -> 27.5
+// ms, 26 (edge factor 16) 7.64 -> 6.68, 24 1.70 -> 1.47, 22 0.51 -> 0.44.
+//
+// A bucket is one word of up to four fields; a field holds the identifying
+// bits of one vertex and, in its top bit, whether this block knows the vertex
+// to be in the tree of name 0. One exact test covers all fields: after the
+// exclusive or with the wanted bits and with every top bit set, subtracting
+// one from each field clears its top bit exactly where the bits agree.
+// Empty fields hold bits of a vertex of the same bucket (or of none below n)
+// and no flag, so they cannot answer wrongly.
+//
+// Flags are learnt in bulk: after its 1st, 2nd, 4th, 8th ... claim a warp
+// looks up its share of the table's vertices. Learning inside the loop, for
+// every lookup that found 0, cost more instructions than the table saved
+// requests (1.74 ms on R-MAT scale 24); only the queue form does it, and only
+// during its first claim, when the hubs have just joined and their lookups
+// would all meet in one L2 sector (rmat 22: 0.49 -> 0.44 ms).
+//
+// kZ: with the zero-tree bitmap. The loop then only reads bits, Q = 4 quads
+// per step, and an edge whose endpoints are not both known goes to the queue as
+// two ids; a full queue loads the parents of 32 edges at once (27.5 ms on R-MAT
+// scale 28 against 28.4 with predicated parent loads in every step).
+// Without Z the parents are the filter, loaded through L2 only, and the next
+// step's edges are loaded ahead (1.52 -> 1.47 ms on R-MAT scale 24; with Z
+// the registers for it cost more than it gave).
+constexpr int kHubBlock = 1024;
+constexpr uint32_t kHubClaimQuads = 1024;  // quads a warp claims at a time (512 and 2048 were slower)
+constexpr size_t kHubSmem = (size_t)(kHubBlock / 32) * 4 * kRing * sizeof(uint32_t) + kWideBuckets * sizeof(uint32_t);
+
+template <bool kZ>
+__global__ void __launch_bounds__(kHubBlock, 1)
+    k_edge_pass_hub(const uint4 *__restrict__ e4, uint64_t n_quads, const uint2 *head, const uint2 *tail, uint32_t *P,
+                    uint32_t n, Ctrl *ctrl, uint32_t *Z, const uint32_t *sel, unsigned long long *work,
+                    const uint32_t *__restrict__ wide, uint32_t s_bits, uint32_t ways) {
+  constexpr int Q = kZ ? 4 : 2;
+  constexpr bool kAhead = !kZ;
+  extern __shared__ uint32_t ring_smem[];
+  if (ld_volatile_u32(sel) == 0u) return;
+  const RootR fn = RootR::load(ctrl);
+  uint32_t *const S = slots<RootR>(P);
+  const uint64_t pol = policy_evict_first();
+  uint32_t *const H = ring_smem;
+  for (uint32_t i = threadIdx.x; i < kWideBuckets / 4; i += kHubBlock)
+    reinterpret_cast<uint4 *>(H)[i] = __ldg(reinterpret_cast<const uint4 *>(wide) + i);
+  WarpRing ring;
+  ring.init(ring_smem + kWideBuckets, nullptr, nullptr, kNeverDirect);
+  const uint32_t fbits = s_bits - kWideBits + 1u;  // field width: identifying bits and flag
+  const uint32_t flag = 1u << (fbits - 1u), rmask = flag - 1u;
+  uint32_t ones = 0;
+  for (uint32_t w = 0; w < ways; ++w) ones |= 1u << (w * fbits);
+  const uint32_t highs = ones * flag;
+  const uint32_t down = 32u - s_bits;
+  const uint32_t mul = kWideMul << down;  // the product's s bits at the top of the word
+  __syncthreads();
+  const uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+  if (t == 0 && head) single_edge(P, fn, head, n, ctrl);
+  if (t == 1 && tail) single_edge(P, fn, tail, n, ctrl);
+  auto load = [&](uint4 (&e)[Q], uint64_t base) {
+#pragma unroll
+    for (int j = 0; j < Q; ++j) {
+      const uint64_t q = base + (uint64_t)j * 32u;
+      e[j] = q < n_quads ? ld_edges_now(e4 + q, pol) : make_uint4(0u, 0u, 0u, 0u);
+    }
+  };
+  // The flag bits of the fields of bucket word `word` that hold y's vertex.
+  auto holds = [&](uint32_t word, uint32_t y) {
+    return ~(((word ^ (((y >> down) & rmask) * ones)) | highs) - ones) & highs;
+  };
+  // kZ: joins `count` queued edges (ids; top bit: known to be in the tree of name 0).
+  auto resolve = [&](uint32_t count) {
+    __syncwarp();
+    const uint32_t slot = (ring.head + ring.lane) & (kRing - 1);
+    const uint32_t xa = ring.cu[slot], xb = ring.cv[slot];
+    __syncwarp();
+    if (ring.lane < count) {
+      const bool ka = xa >> 31, kb = xb >> 31;
+      const uint32_t va = xa & 0x7FFFFFFFu, vb = xb & 0x7FFFFFFFu;
+      uint32_t pa = 0u, pb = 0u;
+      if (!ka) pa = ldP(P + va);
+      if (!kb) pb = ldP(P + vb);
+      bool za = !ka && pa == 0u, zb = !kb && pb == 0u;
+      if (pa != pb) {
+        const UniteResult res = unite(S, fn.f(va), pa, fn.f(vb), pb);
+        za |= res.zero && !ka;
+        zb |= res.zero && !kb;
+      }
+      if (za) zset(Z, fn.f(va));
+      if (zb) zset(Z, fn.f(vb));
+    }
+    ring.head += count;
+  };
+  auto step = [&](uint4 (&e)[Q], bool learning) {
+    uint32_t x[4 * Q], p[4 * Q];  // endpoints; bitmap words (kZ) or parent values
+#pragma unroll
+    for (int j = 0; j < Q; ++j) {
+      if (max(max(e[j].x, e[j].y), max(e[j].z, e[j].w)) >= n) {
+        guard(e[j].x, e[j].y, n, ctrl);
+        guard(e[j].z, e[j].w, n, ctrl);
+      }
+      x[4 * j + 0] = e[j].x;
+      x[4 * j + 1] = e[j].y;
+      x[4 * j + 2] = e[j].z;
+      x[4 * j + 3] = e[j].w;
+    }
+#pragma unroll
+    for (int i = 0; i < 4 * Q; ++i) {
+      const uint32_t y = x[i] * mul;
+      const uint32_t word = H[y >> (32u - kWideBits)];
+      const bool known = (holds(word, y) & word) != 0u;
+      if (kZ) {
+        p[i] = 0xFFFFFFFFu;
+        if (!known) p[i] = ldP(Z + (fn.f(x[i]) >> 5));
+      } else {
+        p[i] = 0u;
+        if (!known) p[i] = ldP_cg(P + x[i]);
+      }
+    }
+    if (!kZ && learning) {
+#pragma unroll
+      for (int i = 0; i < 4 * Q; ++i) {
+        const uint32_t y = x[i] * mul;
+        const uint32_t word = H[y >> (32u - kWideBits)], found = holds(word, y) & ~word;
+        if (p[i] == 0u && found) atomicOr(H + (y >> (32u - kWideBits)), found);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 2 * Q; ++k) {
+      const uint32_t xa = x[2 * k], xb = x[2 * k + 1];
+      if (kZ) {
+        const uint32_t ka = (p[2 * k] >> (fn.f(xa) & 31u)) & 1u, kb = (p[2 * k + 1] >> (fn.f(xb) & 31u)) & 1u;
+        const bool keep = !(ka & kb) && xa != xb;
+        const uint32_t bal = __ballot_sync(0xFFFFFFFFu, keep);
+        if (!bal) continue;
+        if (keep) {
+          const uint32_t slot = (ring.tail + __popc(bal & ring.lt_mask)) & (kRing - 1);
+          ring.cu[slot] = xa | (ka << 31);
+          ring.cv[slot] = xb | (kb << 31);
+        }
+        ring.tail += __popc(bal);
+        if (ring.tail - ring.head >= 32u) resolve(32u);
+      } else {
+        ring.push<true>(S, p[2 * k] != p[2 * k + 1], fn.f(xa), p[2 * k], fn.f(xb), p[2 * k + 1]);
+      }
+    }
+  };
+  constexpr uint32_t kGrab = kHubClaimQuads / (32u * Q);
+  const uint32_t steps = (uint32_t)((n_quads + 32u * Q - 1) / (32u * Q));  // below 2^32 (kHubMaxQuads)
+  for (uint32_t claims = 0;;) {
+    uint32_t g0 = 0;
+    if (ring.lane == 0) g0 = (uint32_t)min(atomicAdd(work, (unsigned long long)kGrab), (unsigned long long)steps);
+    g0 = __shfl_sync(0xFFFFFFFFu, g0, 0);
+    if (g0 >= steps) break;
+    const uint32_t g1 = min(g0 + kGrab, steps);
+    uint4 e[Q];
+    if (kAhead) load(e, (uint64_t)g0 * (32u * Q) + ring.lane);
+    for (uint32_t g = g0; g < g1; ++g) {
+      uint4 cur[Q];
+      if (kAhead) {
+#pragma unroll
+        for (int j = 0; j < Q; ++j) cur[j] = e[j];
+        if (g + 1u < g1) load(e, (uint64_t)(g + 1u) * (32u * Q) + ring.lane);
+      } else {
+        load(cur, (uint64_t)g * (32u * Q) + ring.lane);
+      }
+      step(cur, claims == 0u);
+    }
+    ++claims;
+    if ((claims & (claims - 1u)) == 0u) {
+      constexpr uint32_t kShare = kWideBuckets / (kHubBlock / 32);
+      const uint32_t b0 = (threadIdx.x >> 5) * kShare;
+      for (uint32_t b = b0 + ring.lane; b < b0 + kShare; b += 32u) {
+        const uint32_t word = H[b];
+        uint32_t found = 0u;
+        for (uint32_t w = 0; w < ways; ++w) {
+          const uint32_t f = word >> (w * fbits);
+          const uint32_t v = (((b << (s_bits - kWideBits)) | (f & rmask)) * kWideInv) & (0xFFFFFFFFu >> down);
+          if ((f & flag) || v >= n) continue;
+          if (kZ ? zbit(Z, fn.f(v)) : ldP_cg(P + v) == 0u) found |= flag << (w * fbits);
+        }
+        if (found) atomicOr(H + b, found);
+      }
+    }
+  }
+  if (kZ) {
+    if (ring.tail != ring.head) resolve(ring.tail - ring.head);
+  } else {
+    ring.drain<true>(S);
+  }
+}
+
 __global__ void __launch_bounds__(256) k_validate(const uint4 *__restrict__ e4, uint64_t n_quads,
                                                   const uint2 *head, const uint2 *tail, uint32_t n,
                                                   Ctrl *ctrl, uint32_t *reject) {
@@ -681,6 +880,10 @@ constexpr uint64_t kMinWaves = 8;
 // The queue form reads P through L2 only from this many vertices up (16 MB).
 constexpr uint32_t kL2MinVertices = 1u << 22;
 
+// The wide hot-vertex table pays from about 2^23 edges up: copying it costs a
+// block 128 KB, and below that a warp has at most one claim to learn from.
+constexpr uint64_t kHubMinQuads = 1ULL << 22, kHubMaxQuads = 1ULL << 37;
+
 // Claim size of the dynamic schedule, in warp steps. From 2^20 edges up,
 // 16 steps at a time (measured best there: fewer warps start on the hub's
 // trees at once, so fewer CAS collide). Below that, a smaller graph would
@@ -698,7 +901,8 @@ uint32_t grab_for(uint64_t n_quads, int Q, unsigned grid, int block) {
 template <class F, int Q>
 cudaError_t edge_pass_q(int filter, int block, const EdgeSpan &e, uint32_t *P, uint32_t n, Ctrl *ctrl,
                         const uint32_t *skip, uint32_t *Z, const uint32_t *zsel, bool one_shot, uint32_t *log,
-                        const uint32_t *hub, bool dyn, cudaStream_t s, const unsigned long long *hot) {
+                        const uint32_t *hub, bool dyn, cudaStream_t s, const unsigned long long *hot,
+                        const WideHot *wide_hot) {
   const uint64_t per_block = (uint64_t)block * Q;
   // At least kMinWaves grid iterations per thread: when a whole graph fits
   // one wave, every edge reads P before any hooking and duplicate hub edges
@@ -722,15 +926,31 @@ cudaError_t edge_pass_q(int filter, int block, const EdgeSpan &e, uint32_t *P, u
     const size_t smem_hub = smem + (F::kRF && hot ? kHot * sizeof(uint32_t) : 0);
     // the certificate word chooses among the launched instances (see
     // k_edge_pass_filtered); zsel: with Z, hub: without it
-    if (Z) {
+    const uint32_t *wsel = Z ? zsel : hub;
+    if (F::kRF && wide_hot && wsel && work && !log && !skip && !one_shot && e.n_quads >= kHubMinQuads &&
+        e.n_quads < kHubMaxQuads) {
+      const uint32_t sb = id_bits(n);
+      const void *k = Z ? (const void *)k_edge_pass_hub<true> : (const void *)k_edge_pass_hub<false>;
+      static std::atomic<unsigned long long> set_z{0}, set_p{0};
+      const cudaError_t err =
+          ensure_func_attr(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHubSmem, Z ? set_z : set_p);
+      if (err != cudaSuccess) return err;
+      const unsigned g = (unsigned)persistent_cap(k, kHubBlock, kHubSmem);
+      if (Z)
+        k_edge_pass_hub<true><<<g, kHubBlock, kHubSmem, s>>>(e.quads, e.n_quads, e.head, e.tail, P, n, ctrl, Z, wsel,
+                                                             work, wide_hot->word, sb, wide_ways(sb));
+      else
+        k_edge_pass_hub<false><<<g, kHubBlock, kHubSmem, s>>>(e.quads, e.n_quads, e.head, e.tail, P, n, ctrl, nullptr,
+                                                              wsel, work, wide_hot->word, sb, wide_ways(sb));
+      note_launch();
+    } else if (Z) {
       const void *k = (const void *)k_edge_pass_filtered<F, Q, true, true>;
       const unsigned g = clamp_grid(want, one_shot ? cap_big : persistent_cap(k, block, smem_hub));
       const uint32_t grab = grab_for(e.n_quads, Q, g, block);
       k_edge_pass_filtered<F, Q, true, true><<<g, block, smem_hub, s>>>(e.quads, e.n_quads, e.head, e.tail, P, n,
                                                                         ctrl, skip, Z, zsel, log, work, grab, hot);
       note_launch();
-    }
-    if (!Z && hub) {
+    } else if (hub) {
       const bool l2 = n >= kL2MinVertices;
       const void *k = l2 ? (const void *)k_edge_pass_filtered<F, Q, false, false, true>
                          : (const void *)k_edge_pass_filtered<F, Q, false, false, false>;
@@ -765,11 +985,12 @@ cudaError_t edge_pass_q(int filter, int block, const EdgeSpan &e, uint32_t *P, u
 template <class F>
 cudaError_t edge_pass_f(int filter, int ept, int block, const EdgeSpan &e, uint32_t *P, uint32_t n,
                         Ctrl *ctrl, const uint32_t *skip, uint32_t *Z, const uint32_t *zsel, bool one_shot,
-                        uint32_t *log, const uint32_t *hub, bool dyn, cudaStream_t s, const unsigned long long *hot) {
+                        uint32_t *log, const uint32_t *hub, bool dyn, cudaStream_t s, const unsigned long long *hot,
+                        const WideHot *wide_hot) {
   switch (ept) {
-    case 2: return edge_pass_q<F, 1>(filter, block, e, P, n, ctrl, skip, Z, zsel, one_shot, log, hub, dyn, s, hot);
-    case 8: return edge_pass_q<F, 4>(filter, block, e, P, n, ctrl, skip, Z, zsel, one_shot, log, hub, dyn, s, hot);
-    default: return edge_pass_q<F, 2>(filter, block, e, P, n, ctrl, skip, Z, zsel, one_shot, log, hub, dyn, s, hot);
+    case 2: return edge_pass_q<F, 1>(filter, block, e, P, n, ctrl, skip, Z, zsel, one_shot, log, hub, dyn, s, hot, nullptr);
+    case 8: return edge_pass_q<F, 4>(filter, block, e, P, n, ctrl, skip, Z, zsel, one_shot, log, hub, dyn, s, hot, nullptr);
+    default: return edge_pass_q<F, 2>(filter, block, e, P, n, ctrl, skip, Z, zsel, one_shot, log, hub, dyn, s, hot, wide_hot);
   }
 }
 }  // namespace
@@ -777,13 +998,14 @@ cudaError_t edge_pass_f(int filter, int ept, int block, const EdgeSpan &e, uint3
 cudaError_t launch_edge_pass(bool rf, int filter, int ept, int block, const EdgeSpan &e, uint32_t *P,
                              uint32_t n, Ctrl *ctrl, const uint32_t *skip, cudaStream_t s, uint32_t *Z,
                              const uint32_t *zsel, bool one_shot, uint32_t *log, const uint32_t *hub, bool dyn,
-                             const unsigned long long *hot) {
+                             const unsigned long long *hot, const WideHot *wide_hot) {
   if (block != 128 && block != 256 && block != 512) block = 256;
   if (e.n_quads == 0 && !e.head && !e.tail) return cudaSuccess;
   if (log) filter = 1;  // the log is kept by the filtered form
-  return rf ? edge_pass_f<RootR>(filter, ept, block, e, P, n, ctrl, skip, Z, zsel, one_shot, log, hub, dyn, s, hot)
+  return rf ? edge_pass_f<RootR>(filter, ept, block, e, P, n, ctrl, skip, Z, zsel, one_shot, log, hub, dyn, s, hot,
+                                   wide_hot)
             : edge_pass_f<RootId>(filter, ept, block, e, P, n, ctrl, skip, Z, zsel, one_shot, log, hub, dyn, s,
-                                  nullptr);
+                                  nullptr, nullptr);
 }
 
 cudaError_t launch_validate(const EdgeSpan &e, uint32_t n, Ctrl *ctrl, cudaStream_t s, uint32_t *reject) {

@@ -99,14 +99,15 @@ __global__ void __launch_bounds__(256) k_degree(const uint4 *__restrict__ e4, ui
 __global__ void __launch_bounds__(256) k_degree_sampled(const uint2 *__restrict__ e, uint64_t n_edges,
                                                         uint64_t edge_base, uint32_t stride,
                                                         uint32_t *__restrict__ cnt, uint32_t n, Ctrl *track,
-                                                        uint32_t *list, unsigned int *list_n, uint32_t list_cap) {
+                                                        uint32_t *list, unsigned int *list_n, uint32_t list_cap,
+                                                        uint32_t list_thr) {
   uint32_t top = 0;
   const uint32_t seg = blockIdx.x % kListSegs, seg_room = list_cap / kListSegs;
   auto bump = [&](uint32_t v) {
     if (v >= n) return;
     const uint32_t c = atomicAdd(cnt + v, 1u) + 1u;
     top = max(top, c);
-    if (c == kListThr) {
+    if (c == list_thr) {
       const unsigned int i = atomicAdd(list_n + seg, 1u);
       if (i < seg_room) list[seg * seg_room + i] = v;
     }
@@ -132,8 +133,15 @@ __global__ void __launch_bounds__(256) k_degree_sampled(const uint2 *__restrict_
     }
   }
   if (track) {
+    // one global atomic per block: one per warp meets on the one address for
+    // longer than the sample takes (R-MAT scale 20: 10.3 -> 7 us)
+    __shared__ uint32_t s_top;
+    if (threadIdx.x == 0) s_top = 0u;
+    __syncthreads();
     top = __reduce_max_sync(0xFFFFFFFFu, top);
-    if ((threadIdx.x & 31) == 0 && top) atomicMax(&track->maxkey, (unsigned long long)top << 32);
+    if ((threadIdx.x & 31) == 0 && top) atomicMax(&s_top, top);
+    __syncthreads();
+    if (threadIdx.x == 0 && s_top) atomicMax(&track->maxkey, (unsigned long long)s_top << 32);
   }
 }
 
@@ -212,7 +220,8 @@ static_assert(kCertBuckets == 8192, "13-bit buckets");
 template <bool kList>
 __global__ void __launch_bounds__(256) k_select_candidates(const uint32_t *__restrict__ cnt, uint32_t n,
                                                            Ctrl *ctrl, CertScratch *cs,
-                                                           const uint32_t *__restrict__ list, uint32_t list_cap) {
+                                                           const uint32_t *__restrict__ list, uint32_t list_cap,
+                                                           WideHot *wide_hot, uint32_t s_bits, uint32_t ways) {
   const uint32_t cmax = (uint32_t)(*(volatile unsigned long long *)&ctrl->maxkey >> 32);
   if (cmax < 64u) return;  // uniform over the grid: no block ranks, top stays empty
   const uint32_t thr = cmax >> 5;
@@ -222,33 +231,41 @@ __global__ void __launch_bounds__(256) k_select_candidates(const uint32_t *__res
   // 1.75 ms, 1/128 to 1/2048 1.70 ms).
   const uint32_t hot_thr = cmax >> 8;
   const int lane = threadIdx.x & 31;
-  const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
-  const uint64_t w0 = blockIdx.x * (uint64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
-  const uint64_t count = kList ? list_cap : n;
+  // kList: block b takes segments b, b + gridDim.x, ... and reads only what
+  // they hold; else the grid strides over all vertices
   const uint32_t seg_room = kList ? list_cap / kListSegs : 0u;
-  for (uint64_t base = w0 * 32; base < count; base += warps * 32) {
-    const uint64_t i = base + (uint64_t)lane;
-    bool have = i < count;
-    uint64_t v = i;
-    if constexpr (kList) {
-      if (have) {
-        const uint32_t seg = (uint32_t)(i / seg_room), k = (uint32_t)(i % seg_room);
-        have = k < __ldcg(&cs->list_n[seg]);
-        v = have ? list[i] : 0u;
+  const uint32_t n_rows = kList ? kListSegs : 1u;
+  for (uint32_t row = kList ? blockIdx.x : 0u; row < n_rows; row += kList ? gridDim.x : 1u) {
+    const uint64_t count = kList ? min(__ldcg(&cs->list_n[row]), seg_room) : n;
+    const uint64_t stride = kList ? blockDim.x : (uint64_t)gridDim.x * blockDim.x;
+    const uint64_t first = (kList ? 0u : blockIdx.x * (uint64_t)blockDim.x) + (threadIdx.x & ~31u);
+    for (uint64_t base = first; base < count; base += stride) {
+      const uint64_t i = base + (uint64_t)lane;
+      const bool have = i < count;
+      uint64_t v = i;
+      if constexpr (kList) v = have ? list[(uint64_t)row * seg_room + i] : 0u;
+      const uint32_t c = have ? cnt[v] : 0u;
+      if (c >= hot_thr && c != 0u)
+        atomicMax(&cs->hot[hot_slot((uint32_t)v)], ((unsigned long long)c << 32) | (uint32_t)(v + 1u));
+      if (wide_hot && c != 0u) {
+        // the displaced entry moves on to the next way, so a bucket keeps its best
+        const uint32_t b = wide_bucket(wide_mix((uint32_t)v), s_bits);
+        unsigned long long cur = ((unsigned long long)c << 32) | (uint32_t)(v + 1u);
+        for (uint32_t w = 0; w < ways && cur; ++w) {
+          const unsigned long long old = atomicMax(&wide_hot->slot[w][b], cur);
+          cur = old < cur ? old : cur;
+        }
       }
+      const bool q = c >= thr && c != 0u;
+      const uint32_t bal = __ballot_sync(0xFFFFFFFFu, q);
+      if (!bal) continue;
+      uint32_t seen = 0;
+      if (lane == 0) seen = atomicAdd(&ctrl->n_cand, (uint32_t)__popc(bal)) + (uint32_t)__popc(bal);
+      seen = __shfl_sync(0xFFFFFFFFu, seen, 0);
+      if (seen > kCertCand) break;  // too many candidates (warp-uniform)
+      if (q)
+        atomicMax(&cs->owner[bucket_of((uint32_t)v)], ((unsigned long long)c << 32) | (uint32_t)~(uint32_t)v);
     }
-    const uint32_t c = have ? cnt[v] : 0u;
-    if (c >= hot_thr && c != 0u)
-      atomicMax(&cs->hot[hot_slot((uint32_t)v)], ((unsigned long long)c << 32) | (uint32_t)(v + 1u));
-    const bool q = c >= thr && c != 0u;
-    const uint32_t bal = __ballot_sync(0xFFFFFFFFu, q);
-    if (!bal) continue;
-    uint32_t seen = 0;
-    if (lane == 0) seen = atomicAdd(&ctrl->n_cand, (uint32_t)__popc(bal)) + (uint32_t)__popc(bal);
-    seen = __shfl_sync(0xFFFFFFFFu, seen, 0);
-    if (seen > kCertCand) break;  // too many candidates (warp-uniform)
-    if (q)
-      atomicMax(&cs->owner[bucket_of((uint32_t)v)], ((unsigned long long)c << 32) | (uint32_t)~(uint32_t)v);
   }
   __shared__ unsigned s_last;
   __threadfence();
@@ -283,6 +300,18 @@ __global__ void __launch_bounds__(256) k_select_candidates(const uint32_t *__res
     if (threadIdx.x == 0) cs->top[r] = best;
     if (mine == best) ++next;
   }
+}
+
+// Packs the buckets of the wide hot-vertex table, one thread each.
+__global__ void __launch_bounds__(256) k_wide_hot_pack(WideHot *h, uint32_t s_bits, uint32_t ways) {
+  const uint32_t b = blockIdx.x * blockDim.x + threadIdx.x;
+  const uint32_t rbits = s_bits - kWideBits;
+  uint32_t word = 0;
+  for (uint32_t w = 0; w < ways; ++w) {
+    const uint32_t x1 = (uint32_t)h->slot[w][b];
+    if (x1) word |= (wide_mix(x1 - 1u) & ((1u << rbits) - 1u)) << (w * (rbits + 1u));
+  }
+  h->word[b] = word;
 }
 
 constexpr size_t kCertSmem = kCertBuckets * sizeof(uint32_t);  // 32 KiB
@@ -535,12 +564,13 @@ cudaError_t launch_degree_u32(const EdgeSpan &e, uint32_t *cnt, uint32_t n, cuda
 
 cudaError_t launch_degree_sampled_u32(const uint2 *edges, uint64_t n_edges, uint64_t edge_base,
                                       uint32_t stride, uint32_t *cnt, uint32_t n, cudaStream_t s, Ctrl *track,
-                                      uint32_t *list, unsigned int *list_n, uint32_t list_cap) {
+                                      uint32_t *list, unsigned int *list_n, uint32_t list_cap, uint32_t list_thr) {
   if (n_edges == 0) return cudaSuccess;
   if (stride == 0) stride = 1;
   const uint64_t groups = ((n_edges + kSampleGroup - 1) >> kSampleGroupShift) / stride + 2;
   const unsigned g = clamp_grid(groups * kSampleGroup / 256, persistent_cap((const void *)k_degree_sampled, 256, 0));
-  k_degree_sampled<<<g, 256, 0, s>>>(edges, n_edges, edge_base, stride, cnt, n, track, list, list_n, list_cap);
+  k_degree_sampled<<<g, 256, 0, s>>>(edges, n_edges, edge_base, stride, cnt, n, track, list, list_n, list_cap,
+                                       list_thr);
   note_launch();
   return cudaGetLastError();
 }
@@ -555,8 +585,9 @@ cudaError_t launch_argmax_u32(const uint32_t *cnt, uint32_t n, Ctrl *ctrl, cudaS
 cudaError_t launch_root_select_certified(const uint32_t *edges, uint64_t n_edges, const EdgeSpan &e,
                                          void *cnt, bool wide, uint32_t n, CertScratch *cs, Ctrl *ctrl,
                                          cudaStream_t s, uint32_t *push_buf, uint32_t push_cap,
-                                         uint32_t *list, uint32_t list_cap) {
+                                         uint32_t *list, uint32_t list_cap, WideHot *wide_hot) {
   cudaError_t err;
+  const uint32_t s_bits = id_bits(n);
   if (!list || list_cap < kListSegs || list_cap % kListSegs) list = nullptr;
   // 0. reset the sampled counters, the scratch and the control fields
   if ((err = cudaMemsetAsync(cnt, 0, (size_t)n * sizeof(uint32_t), s)) != cudaSuccess) return err;
@@ -564,25 +595,31 @@ cudaError_t launch_root_select_certified(const uint32_t *edges, uint64_t n_edges
   if ((err = cudaMemsetAsync(&ctrl->maxkey, 0, 2 * sizeof(unsigned long long), s)) != cudaSuccess) return err;
   if ((err = cudaMemsetAsync(&ctrl->m_sel, 0xFF, sizeof(uint32_t), s)) != cudaSuccess) return err;
   if ((err = cudaMemsetAsync(&ctrl->n_cand, 0, 2 * sizeof(uint32_t), s)) != cudaSuccess) return err;
+  if (!list) wide_hot = nullptr;
+  if (wide_hot && (err = cudaMemsetAsync(wide_hot->slot, 0, wide_ways(s_bits) * sizeof(wide_hot->slot[0]), s)) != cudaSuccess) return err;
   uint32_t *c32 = static_cast<uint32_t *>(cnt);
   // 1. sampled histogram and its largest count; the push list also needs the
   // vertex holding it (the argmax pass)
   const uint32_t stride = cert_sample_stride(n_edges);
   if ((err = launch_degree_sampled_u32(reinterpret_cast<const uint2 *>(edges), n_edges, 0, stride, c32, n, s,
-                                       push_buf ? nullptr : ctrl, list, cs->list_n, list_cap)) != cudaSuccess)
+                                       push_buf ? nullptr : ctrl, list, cs->list_n, list_cap,
+                                       wide_hot ? kWideListThr : kListThr)) != cudaSuccess)
     return err;
   if (push_buf && (err = launch_argmax_u32(c32, n, ctrl, s)) != cudaSuccess) return err;
   // 2. candidates: the owners of their buckets, from the list when there is one
   if (list) {
-    const unsigned gsel = clamp_grid(((uint64_t)list_cap + 255) / 256,
-                                     persistent_cap((const void *)k_select_candidates<true>, 256, 0));
-    k_select_candidates<true><<<gsel, 256, 0, s>>>(c32, n, ctrl, cs, list, list_cap);
+    k_select_candidates<true><<<kListSegs, 256, 0, s>>>(c32, n, ctrl, cs, list, list_cap, wide_hot,
+                                                s_bits, wide_hot ? wide_ways(s_bits) : 0u);
   } else {
     const unsigned gsel = clamp_grid(((uint64_t)n + 255) / 256,
                                      persistent_cap((const void *)k_select_candidates<false>, 256, 0));
-    k_select_candidates<false><<<gsel, 256, 0, s>>>(c32, n, ctrl, cs, nullptr, 0u);
+    k_select_candidates<false><<<gsel, 256, 0, s>>>(c32, n, ctrl, cs, nullptr, 0u, nullptr, 0u, 0u);
   }
   note_launch();
+  if (wide_hot) {
+    k_wide_hot_pack<<<kWideBuckets / 256, 256, 0, s>>>(wide_hot, s_bits, wide_ways(s_bits));
+    note_launch();
+  }
   // 3. the exact pass in shared memory
   static std::atomic<unsigned long long> smem_set_certify{0};
   if ((err = ensure_func_attr((const void *)k_degree_certify, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -687,7 +724,7 @@ cudaError_t chunked_select_begin(const uint32_t *chunk0, uint64_t n0, void *cnt,
   if ((err = launch_argmax_u32(c32, n, ctrl, s)) != cudaSuccess) return err;
   const unsigned gsel = clamp_grid(((uint64_t)n + 255) / 256,
                                    persistent_cap((const void *)k_select_candidates<false>, 256, 0));
-  k_select_candidates<false><<<gsel, 256, 0, s>>>(c32, n, ctrl, cs, nullptr, 0u);
+  k_select_candidates<false><<<gsel, 256, 0, s>>>(c32, n, ctrl, cs, nullptr, 0u, nullptr, 0u, 0u);
   note_launch();
   k_spec_begin<<<1, 1, 0, s>>>(ctrl);
   note_launch();
