@@ -1014,7 +1014,7 @@ def bench_batched(args, cc, graphgen, torch, stream):
                          "algorithmic_bytes_per_launch": alg,
                          "algorithmic_bytes": "8 B per edge + 12 B per vertex (init write, compression "
                                               "read, label write)",
-                         "kernel": "k_batched, one launch per replay; time = median replay (CUDA events)",
+                         "kernel": "the k_batch_* launches of a replay; time = median replay (CUDA events)",
                          "peak_source": f"{peak_kind} (HBM copy bandwidth)"}}
 
 

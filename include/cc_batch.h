@@ -1,6 +1,6 @@
 /*
  * cc_batch.h - connected components of many independent graphs in one
- * launch (C ABI; conventions as in cc.h).
+ * call (C ABI; conventions as in cc.h).
  *
  * Graph g owns vertices [vtx_off[g], vtx_off[g+1]) and edges
  * [edge_off[g], edge_off[g+1]) of one concatenated edge list whose ids are
@@ -10,13 +10,14 @@
  *
  * Method: Algorithm 1 (Root-Function JT with f(v) = v) on the union of all
  * graphs, whose vertex sets occupy disjoint ranges of one name space, so the
- * forests of different graphs never meet. One cooperative persistent kernel
- * runs the phases (tile offsets, initialisation, hooking over edge tiles that
- * each lie inside one graph, compression, local labels) separated by grid
- * barriers whose waits are bounded; the label array doubles as the parent
- * array, so a run allocates nothing. The launch can be captured in a CUDA
- * graph. The tile size, block size, edges per thread and the warp filter are
- * chosen by cc_batch_tune.
+ * forests of different graphs never meet. The phases are a few launches on the
+ * caller's stream, all covering every graph: tile offsets and initialisation
+ * (cooperative, with one grid barrier whose wait is bounded), hooking over
+ * edge tiles that each lie inside one graph, compression, the edges that
+ * hooking left over, compression, local labels. The label array doubles as the
+ * parent array, so a run allocates nothing. The launches can be captured in a
+ * CUDA graph. The tile size, block size, edges per thread and the warp filter
+ * of the hooking are chosen by cc_batch_tune.
  */
 #ifndef CC_BATCH_H
 #define CC_BATCH_H
@@ -37,9 +38,11 @@ typedef struct cc_batch_config {
   int32_t block_size;       /* 256 or 512 */
   int32_t edges_per_thread; /* 1, 2 or 4 per round */
   int32_t filter;           /* 1: warp filter + compaction, 0: per-lane */
-  uint32_t tile_edges;      /* edges per hooking tile (one warp's unit of work), a multiple of 256, >= 256 */
+  uint32_t tile_edges;      /* edges per hooking tile (one warp's unit of work), a multiple of 256, >= 256;
+                               3/8 of them are hooked in the first phase, and small batches use
+                               smaller tiles, so that every warp has some */
   uint32_t tile_vertices;   /* vertices per tile of the label phase, >= 256 */
-  uint32_t barrier_wait_us; /* bounded wait of each grid barrier, at most 60 s; 0 = 4 s. A
+  uint32_t barrier_wait_us; /* bounded wait of the grid barrier, at most 60 s; 0 = 4 s. A
                                wait that expires aborts the run (every block leaves at its
                                next barrier; the labels are then undefined) and cc_batch_sync
                                returns CC_ERR_TIMEOUT; the next run starts afresh. The
@@ -48,7 +51,7 @@ typedef struct cc_batch_config {
 } cc_batch_config;
 
 /* A batch context for up to max_graphs graphs per call: its tile-offset
- * scratch (16 bytes per graph) and control block. */
+ * scratch (28 bytes per graph) and control block. */
 CC_API cc_status cc_batch_create(uint32_t max_graphs, cc_batch **out);
 
 /* Labels of n_graphs graphs (n_graphs <= max_graphs). vtx_off_dev and

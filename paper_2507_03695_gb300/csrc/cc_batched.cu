@@ -1,18 +1,30 @@
 // cc_batched.cu - connected components of many independent graphs in one
-// cooperative persistent launch (include/cc_batch.h).
+// call (include/cc_batch.h).
 //
 // All graphs share one name space: vertex i of graph g is named
 // vtx_off[g] + i and f is the identity (Algorithm 1), so each graph's forest
 // lives in its own range and the root of a component is its smallest global
 // name; minus vtx_off[g] that is the graph-local min-id label. The label array
-// is the parent array during the run. Phases, separated by grid barriers:
-//   0. block 0 checks the offsets and turns them into tile offsets;
-//   1. P[x] = x for every vertex;
-//   2. hooking: edge tiles (each inside one graph) with rebased ids, through
-//      the warp ring or per lane;
-//   3. compression: every vertex stores its root's name (read-only walks with
-//      L2-coherent loads, so each entry is written only by its owner);
-//   4. labels: vertex tiles turn root names into graph-local ids in place.
+// is the parent array during the run. Phases, each a launch of its own so that
+// each has the registers and shared memory it needs (as one kernel the hooking
+// ran at half its occupancy):
+//   0. one block checks the offsets and turns them into tile offsets; after a
+//      grid barrier every vertex gets P[x] = x (k_batch_begin, cooperative);
+//   1. hooking: edge tiles (each inside one graph) through the warp ring or
+//      per lane; of a graph with many edges per vertex only one chunk in
+//      sample_stride, which is enough to form its giant component;
+//   2. compression: every vertex stores its root's name, and each sampled
+//      graph gets a reference, the root that most of its vertices have;
+//   3. the chunks left over, against one bit per vertex in shared memory: an
+//      edge inside the reference's tree costs two shared-memory loads;
+//   4. compression;
+//   5. labels: vertex tiles turn root names into graph-local ids in place.
+// Measured in ms, before (every edge hooked, one cooperative kernel) and now:
+// 4096 mixed graphs (1.18G edges) 12.2 -> 8.5, 400 graphs 2.0 -> 1.4, 40
+// graphs 0.89 -> 0.49, one graph of 38K edges 0.39 -> 0.08. Of 2000 graphs'
+// 3.8 ms phases 0 to 5 take 0.06 / 2.0 / 0.27 / 1.2 / 0.09 / 0.18: phase 1
+// waits for the dependent loads and compare-and-swaps of the searches, phase 3
+// issues 3.3 instructions per clock.
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <string.h>
@@ -31,7 +43,8 @@ struct alignas(128) BatchCtrl {
   unsigned int abort;        // nonzero: every block leaves at the next barrier } each run
   unsigned int err;          // kErr* bits (sticky until cc_batch_sync)
   unsigned int bad_offsets;  // malformed offsets (sticky until cc_batch_sync)
-  unsigned int pad[3];
+  unsigned int tile_chunks;  // chunks per hooking tile of this run
+  unsigned long long segs;   // segments of the filtered phase claimed so far (reset before each run)
 };
 
 struct BatchArgs {
@@ -42,7 +55,10 @@ struct BatchArgs {
   uint32_t *P;  // the label array
   uint64_t *etile_off;  // n_graphs + 1
   uint64_t *vtile_off;  // n_graphs + 1
+  uint64_t *chunk_off;  // n_graphs + 1: chunks of the graphs that the filtered phase takes
+  uint32_t *ref;        // n_graphs: the root of each such graph's reference tree
   uint32_t tile_edges, tile_vertices;
+  uint32_t hook_warps;  // warps of the hooking launch
   unsigned long long barrier_ns;  // bounded wait of every grid barrier
   BatchCtrl *ctrl;
 };
@@ -56,19 +72,6 @@ __device__ __forceinline__ unsigned long long globaltimer() {
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
 }
-
-// Built with -DCC_BATCH_CLOCK, block 0 records the global timer at the
-// kernel's start, after each grid barrier and at its end (diagnostics of the
-// phase times only, off in normal builds).
-#ifdef CC_BATCH_CLOCK
-__device__ unsigned long long g_batch_clock[8];
-#define CC_BATCH_TICK(i)                                                     \
-  do {                                                                       \
-    if (blockIdx.x == 0 && threadIdx.x == 0) g_batch_clock[(i)] = globaltimer(); \
-  } while (0)
-#else
-#define CC_BATCH_TICK(i) ((void)0)
-#endif
 
 __device__ __forceinline__ unsigned int ld_acquire_u32(const unsigned int *p) {
   unsigned int v;
@@ -110,96 +113,135 @@ __device__ bool grid_barrier(BatchCtrl *c, unsigned int &gen, unsigned long long
   }
   __syncthreads();
   ++gen;
-  CC_BATCH_TICK(gen);
   return s_ok != 0;
 }
 
-// Largest g in [0, n) with off[g] <= t (off nondecreasing, off[0] == 0).
-__device__ __forceinline__ uint32_t owner(const uint64_t *off, uint32_t n, uint64_t t) {
+// Edges are taken in chunks of kChunkEdges, four per lane of a warp.
+constexpr uint32_t kChunkEdges = 128;
+// The filtered phase keeps a bit per vertex of one graph in shared memory: 32
+// KB per block leave room for 48 warps per SM.
+constexpr uint32_t kBitsMax = 1u << 18;
+// Graphs with fewer edges, or fewer than three per vertex, are hooked whole:
+// the sample that forms their giant component would be most of them.
+constexpr uint64_t kFilterMinEdges = 1u << 15;
+constexpr uint64_t kFilterMinDegree = 3;
+constexpr uint64_t kStrideMax = 64;
+
+// One chunk in sample_stride is hooked first; 1: all of them. The sample
+// holds 1.5 edges per vertex: with one per vertex the giant component of a
+// uniform graph is still missing a fifth of the vertices and the filter lets
+// too many edges through (2000 mixed graphs: 4.05 ms with one, 3.91 with 1.5,
+// 4.14 with two).
+__device__ __forceinline__ uint32_t sample_stride(uint64_t n_edges, uint64_t nv) {
+  if (nv == 0 || nv > kBitsMax || n_edges < kFilterMinEdges || n_edges < kFilterMinDegree * nv) return 1u;
+  const uint64_t s = 2 * n_edges / (3 * nv);
+  return (uint32_t)(s < kStrideMax ? s : kStrideMax);
+}
+
+// Largest g in [0, n) with off[g] <= t (off nondecreasing, off[0] == 0), by a
+// whole warp: every lane calls it, 32 candidates per round.
+__device__ __forceinline__ uint32_t owner_warp(const uint64_t *off, uint32_t n, uint64_t t) {
+  const uint32_t lane = threadIdx.x & 31u;
   uint32_t lo = 0, hi = n;  // answer in [lo, hi)
   while (hi - lo > 1u) {
-    const uint32_t mid = (lo + hi) >> 1;
-    if (off[mid] <= t)
-      lo = mid;
-    else
-      hi = mid;
+    const uint32_t step = (hi - lo + 31u) / 32u;
+    const uint64_t i = lo + (uint64_t)lane * step;
+    const uint32_t at_most = __ballot_sync(0xFFFFFFFFu, i < hi && off[i] <= t);  // lane 0 always
+    lo += (31u - (uint32_t)__clz((int)at_most)) * step;
+    hi = hi - lo > step ? lo + step : hi;
   }
   return lo;
+}
+
+// Chunks that a hooking tile holds: 3/8 of the configured tile's (the default
+// 8192 edges: 24 chunks), or fewer where that would leave less than four tiles
+// per warp. Between 15 and 30 chunks 4096 graphs take 8.4 to 8.6 ms, with 61
+// 10.2 (the last tiles leave most warps idle); 400 graphs take 1.37 ms with 6
+// and 1.69 with 2 (a warp's tiles are then of several graphs and share
+// nothing in L1); one graph of 38K edges took 0.39 ms in five tiles of 8192
+// edges and takes 0.08.
+constexpr uint64_t kTilesPerWarp = 4;
+constexpr uint32_t kTileMinChunks = 2;
+
+// Chunks of graph g that phase 1 hooks (0 when its offsets decrease).
+__device__ __forceinline__ uint64_t hooked_chunks(const BatchArgs &a, uint32_t g) {
+  const uint64_t v0 = a.vtx_off[g], v1 = a.vtx_off[g + 1], e0 = a.edge_off[g], e1 = a.edge_off[g + 1];
+  if (v1 < v0 || e1 < e0) return 0;
+  const uint32_t stride = sample_stride(e1 - e0, v1 - v0);
+  return ((e1 - e0 + kChunkEdges - 1) / kChunkEdges + stride - 1) / stride;
 }
 
 // Phase 0 (one block): validate the offsets and write exclusive prefix sums
 // of the per-graph tile counts.
 __device__ void scan_tiles(const BatchArgs &a) {
-  __shared__ unsigned long long s_carry_e, s_carry_v;
-  __shared__ unsigned long long s_we[32], s_wv[32];
+  constexpr int K = 3;  // hooking tiles, vertex tiles, chunks of the filtered phase
+  __shared__ unsigned long long s_carry[K], s_w[K][32];
   __shared__ int s_bad;
-  if (threadIdx.x == 0) {
-    s_carry_e = s_carry_v = 0ULL;
-    s_bad = (a.vtx_off[0] != 0ULL || a.edge_off[0] != 0ULL);
-  }
+  uint64_t *const out[K] = {a.etile_off, a.vtile_off, a.chunk_off};
+  if (threadIdx.x < K) s_carry[threadIdx.x] = 0ULL;
+  if (threadIdx.x == 0) s_bad = (a.vtx_off[0] != 0ULL || a.edge_off[0] != 0ULL);
   __syncthreads();
   const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  // the chunks to hook, all graphs together, and from them a tile's size
+  __shared__ unsigned long long s_hooked;
+  if (threadIdx.x == 0) s_hooked = 0ULL;
+  __syncthreads();
+  unsigned long long hooked = 0;
+  for (uint32_t g = threadIdx.x; g < a.n_graphs; g += blockDim.x) hooked += hooked_chunks(a, g);
+  hooked = warp_sum_u64(hooked);
+  if (lane == 0) atomicAdd(&s_hooked, hooked);
+  __syncthreads();
+  const uint64_t even = s_hooked / (kTilesPerWarp * a.hook_warps);
+  const uint32_t share = a.tile_edges / kChunkEdges * 3u / 8u, most = share > kTileMinChunks ? share : kTileMinChunks;
+  const uint32_t per_tile = even >= most ? most : (even < kTileMinChunks ? kTileMinChunks : (uint32_t)even);
+  if (threadIdx.x == 0) a.ctrl->tile_chunks = per_tile;
   for (uint32_t base = 0; base < a.n_graphs; base += blockDim.x) {
     const uint32_t g = base + threadIdx.x;
-    unsigned long long te = 0, tv = 0;
+    unsigned long long own[K] = {0, 0, 0}, incl[K];
     if (g < a.n_graphs) {
       const uint64_t v0 = a.vtx_off[g], v1 = a.vtx_off[g + 1];
       const uint64_t e0 = a.edge_off[g], e1 = a.edge_off[g + 1];
-      if (v1 < v0 || e1 < e0) s_bad = 1;
-      else {
-        te = (e1 - e0 + a.tile_edges - 1) / a.tile_edges;
-        tv = (v1 - v0 + a.tile_vertices - 1) / a.tile_vertices;
+      if (v1 < v0 || e1 < e0) {
+        s_bad = 1;
+      } else {
+        const uint64_t chunks = (e1 - e0 + kChunkEdges - 1) / kChunkEdges;
+        const uint32_t stride = sample_stride(e1 - e0, v1 - v0);
+        own[0] = ((chunks + stride - 1) / stride + per_tile - 1) / per_tile;
+        own[1] = (v1 - v0 + a.tile_vertices - 1) / a.tile_vertices;
+        own[2] = stride > 1u ? chunks : 0u;
       }
     }
-    // inclusive warp scans
-    unsigned long long ie = te, iv = tv;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned long long ye = __shfl_up_sync(0xFFFFFFFFu, ie, o);
-      const unsigned long long yv = __shfl_up_sync(0xFFFFFFFFu, iv, o);
-      if (lane >= (uint32_t)o) {
-        ie += ye;
-        iv += yv;
-      }
-    }
-    if (lane == 31) {
-      s_we[wid] = ie;
-      s_wv[wid] = iv;
-    }
-    __syncthreads();
-    if (wid == 0) {
-      unsigned long long xe = lane < nw ? s_we[lane] : 0ULL, xv = lane < nw ? s_wv[lane] : 0ULL;
+    for (int k = 0; k < K; ++k) {  // inclusive warp scans
+      incl[k] = own[k];
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long ye = __shfl_up_sync(0xFFFFFFFFu, xe, o);
-        const unsigned long long yv = __shfl_up_sync(0xFFFFFFFFu, xv, o);
-        if (lane >= (uint32_t)o) {
-          xe += ye;
-          xv += yv;
-        }
+        const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, incl[k], o);
+        if (lane >= (uint32_t)o) incl[k] += y;
       }
-      if (lane < nw) {
-        s_we[lane] = xe;  // inclusive prefix over warps
-        s_wv[lane] = xv;
-      }
+      if (lane == 31) s_w[k][wid] = incl[k];
     }
     __syncthreads();
-    const unsigned long long off_e = s_carry_e + (wid ? s_we[wid - 1] : 0ULL) + ie - te;
-    const unsigned long long off_v = s_carry_v + (wid ? s_wv[wid - 1] : 0ULL) + iv - tv;
-    if (g < a.n_graphs) {
-      a.etile_off[g] = off_e;
-      a.vtile_off[g] = off_v;
+    if (wid < K) {  // warp k scans the warp totals of quantity k
+      unsigned long long x = lane < nw ? s_w[wid][lane] : 0ULL;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+        if (lane >= (uint32_t)o) x += y;
+      }
+      __syncwarp();
+      if (lane < nw) s_w[wid][lane] = x;  // inclusive prefix over warps
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-      s_carry_e += s_we[nw - 1];
-      s_carry_v += s_wv[nw - 1];
-    }
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+      if (g < a.n_graphs) out[k][g] = s_carry[k] + (wid ? s_w[k][wid - 1] : 0ULL) + incl[k] - own[k];
+    __syncthreads();
+    if (threadIdx.x < K) s_carry[threadIdx.x] += s_w[threadIdx.x][nw - 1];
     __syncthreads();
   }
+  if (threadIdx.x < K) out[threadIdx.x][a.n_graphs] = s_carry[threadIdx.x];
   if (threadIdx.x == 0) {
-    a.etile_off[a.n_graphs] = s_carry_e;
-    a.vtile_off[a.n_graphs] = s_carry_v;
     if (a.vtx_off[a.n_graphs] > 0x7FFFFFFFULL) s_bad = 1;
     if (s_bad) {
       a.ctrl->bad_offsets = 1u;
@@ -208,28 +250,236 @@ __device__ void scan_tiles(const BatchArgs &a) {
   }
 }
 
-template <int EPT, bool FILTER>
-__global__ void __launch_bounds__(512) k_batched(BatchArgs a) {
-  extern __shared__ uint32_t ring_smem[];
-  __shared__ uint64_t s_tile[4];  // graph, first edge / vertex, end, name base
-  BatchCtrl *c = a.ctrl;
-  unsigned int gen = 0;
-  CC_BATCH_TICK(0);
-  if (blockIdx.x == 0) scan_tiles(a);
-  if (!grid_barrier(c, gen, a.barrier_ns)) return;
+// Root of vertex x by a read-only walk through L2.
+__device__ __forceinline__ uint32_t walk_root(const uint32_t *P, uint32_t x) {
+  uint32_t r = x, pr = ldP_cg(P + r);
+  while (pr != r) {
+    r = pr;
+    pr = ldP_cg(P + r);
+  }
+  return r;
+}
 
-  // 1. initialisation: P[x] = x
+// Every vertex stores its root's name: read-only walks, four per thread in
+// lock step, so that their dependent loads overlap; each entry is written
+// only by its owner.
+__device__ void compress(uint32_t *P, uint64_t V, uint64_t tid, uint64_t T) {
+  const uint64_t head = ((16u - ((uintptr_t)P & 15u)) & 15u) / 4u;  // entries before the first 16-byte boundary
+  const uint64_t h = head < V ? head : V, n4 = (V - h) / 4u;
+  for (uint64_t i = tid; i < n4; i += T) {
+    const uint64_t x0 = h + 4u * i;
+    uint32_t r[4], p[4];
+    asm volatile("ld.global.cg.v4.u32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "l"(P + x0)
+                 : "memory");
+    uint32_t run = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      p[k] = r[k];
+      run |= (uint32_t)(r[k] != (uint32_t)(x0 + k)) << k;
+    }
+    while (run) {
+      uint32_t q[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if ((run >> k) & 1u) q[k] = ldP_cg(P + r[k]);
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if ((run >> k) & 1u) {
+          if (q[k] == r[k]) run &= ~(1u << k);
+          r[k] = q[k];
+        }
+    }
+    if (r[0] != p[0] || r[1] != p[1] || r[2] != p[2] || r[3] != p[3])
+      *reinterpret_cast<uint4 *>(P + x0) = make_uint4(r[0], r[1], r[2], r[3]);
+  }
+  const uint64_t rest = V - 4u * n4;  // the entries before and after the aligned body
+  if (tid < rest) {
+    const uint64_t x = tid < h ? tid : tid + 4u * n4;
+    const uint32_t px = ldP_cg(P + x), r = walk_root(P, px);
+    if (r != px) stP(P + x, r);
+  }
+}
+
+// Segments of consecutive chunks per block, claimed from a counter: more
+// segments balance better, but each starts by building its graph's bits (2000
+// mixed graphs, this phase: 1.24, 1.27 and 1.68 ms with 4, 8 and 16).
+constexpr uint32_t kSegs = 4;
+
+// The filtered phase: the chunks of each graph that the hooking phase left,
+// against one bit per vertex in shared memory, set for the members of the
+// graph's reference tree.
+__device__ void filtered_phase(const BatchArgs &a, uint32_t *bits, uint32_t *ring_words) {
+  __shared__ unsigned long long s_claim;
+  __shared__ uint32_t s_graph;
+  BatchCtrl *const c = a.ctrl;
+  uint32_t *const P = a.P;
+  const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const uint32_t lt_mask = (1u << lane) - 1u;
+  // a queue of ids per warp: a's id in the first half, b's in the second
+  uint32_t *const qa = ring_words + wid * 2 * kRing, *const qb = qa + kRing;
+  const uint64_t total = a.chunk_off[a.n_graphs];
+  if (total == 0) return;
+  uint64_t seg = (total + (uint64_t)gridDim.x * kSegs - 1) / ((uint64_t)gridDim.x * kSegs);
+  if (seg < 64) seg = 64;
+  uint32_t built = 0xFFFFFFFFu;  // the graph whose bits are in shared memory
+  for (;;) {
+    if (threadIdx.x == 0) s_claim = atomicAdd(&c->segs, 1ULL);
+    __syncthreads();
+    uint64_t t = s_claim * seg;
+    const uint64_t t1 = t + seg < total ? t + seg : total;
+    if (t >= total) return;
+    while (t < t1) {
+      if (wid == 0) {
+        const uint32_t found = owner_warp(a.chunk_off, a.n_graphs, t);
+        if (lane == 0) s_graph = found;
+      }
+      __syncthreads();
+      const uint32_t g = s_graph;
+      const uint64_t base64 = a.vtx_off[g];
+      const uint32_t base = (uint32_t)base64, nv = (uint32_t)(a.vtx_off[g + 1] - base64);
+      const uint64_t e0 = a.edge_off[g], n_e = a.edge_off[g + 1] - e0;
+      const uint32_t c0 = (uint32_t)(t - a.chunk_off[g]);
+      const uint64_t t_end = a.chunk_off[g + 1] < t1 ? a.chunk_off[g + 1] : t1;
+      const uint32_t c1 = (uint32_t)(t_end - a.chunk_off[g]);
+      t = t_end;
+      const uint32_t stride = sample_stride(n_e, nv);
+      const uint32_t ref = a.ref[g];
+      if (built != g) {
+        const uint32_t words = (nv + 31u) / 32u;
+        for (uint32_t w0 = wid * 4u; w0 < words; w0 += nw * 4u) {
+          uint32_t p[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const uint32_t v = (w0 + k) * 32u + lane;
+            p[k] = v < nv ? ldP_cg(P + base + v) : ~ref;
+          }
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const uint32_t word = __ballot_sync(0xFFFFFFFFu, p[k] == ref);
+            if (lane == 0 && w0 + k < words) bits[w0 + k] = word;
+          }
+        }
+        built = g;
+        __syncthreads();
+      }
+      uint32_t head = 0, tail = 0;
+      auto resolve = [&](uint32_t count) {
+        __syncwarp();
+        const uint32_t slot = (head + lane) & (kRing - 1);
+        const uint32_t xa = qa[slot], xb = qb[slot];
+        __syncwarp();
+        if (lane < count) {
+          const uint32_t va = xa & 0x7FFFFFFFu, vb = xb & 0x7FFFFFFFu;
+          uint32_t pa = ref, pb = ref;  // a marked endpoint's parent was ref once
+          if (!(xa >> 31)) pa = ldP_cg(P + base + va);
+          if (!(xb >> 31)) pb = ldP_cg(P + base + vb);
+          if (!(xa >> 31) && pa == ref) atomicOr(bits + (va >> 5), 1u << (va & 31u));
+          if (!(xb >> 31) && pb == ref) atomicOr(bits + (vb >> 5), 1u << (vb & 31u));
+          if (pa != pb) unite<true>(P, base + va, pa, base + vb, pb);
+        }
+        head += count;
+      };
+      // this warp's chunks that were not sampled, the next one loaded ahead
+      const uint32_t full = (uint32_t)(n_e / kChunkEdges);  // chunks before a ragged last one
+      const uint2 *const e_lane = a.edges + e0 + lane;
+      const uint32_t hop = nw % stride;
+      uint32_t ch = c0 + wid, phase = ch % stride;
+      auto skip = [&]() {
+        while (phase == 0u && ch < c1) {
+          ch += nw;
+          phase = hop;
+        }
+      };
+      uint2 e[4];
+      auto load = [&]() {
+        const uint2 *const p = e_lane + (uint64_t)ch * kChunkEdges;
+        if (ch < full) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) e[j] = ld_edge_now(p + 32 * j);
+        } else {
+          const uint32_t left = (uint32_t)(n_e - (uint64_t)ch * kChunkEdges);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            e[j] = make_uint2(0u, 0u);
+            if (lane + 32u * j < left) e[j] = ld_edge_now(p + 32 * j);
+          }
+        }
+      };
+      skip();
+      if (ch < c1) load();
+      while (ch < c1) {
+        uint2 cur[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) cur[j] = e[j];
+        ch += nw;
+        phase += hop;
+        if (phase >= stride) phase -= stride;
+        skip();
+        if (ch < c1) load();
+        const uint32_t top = max(max(max(cur[0].x, cur[0].y), max(cur[1].x, cur[1].y)),
+                                 max(max(cur[2].x, cur[2].y), max(cur[3].x, cur[3].y)));
+        if (top >= nv) {
+          atomicOr(&c->err, kErrRange);
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (max(cur[j].x, cur[j].y) >= nv) cur[j] = make_uint2(0u, 0u);
+        }
+        uint32_t wa[4], wb[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          wa[j] = bits[cur[j].x >> 5];
+          wb[j] = bits[cur[j].y >> 5];
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          // the vertex's bit comes to the bottom (the rotation takes the count modulo 32)
+          const uint32_t ka = __funnelshift_r(wa[j], wa[j], cur[j].x), kb = __funnelshift_r(wb[j], wb[j], cur[j].y);
+          const bool keep = !(ka & kb & 1u);
+          const uint32_t bal = __ballot_sync(0xFFFFFFFFu, keep);
+          if (!bal) continue;
+          if (keep) {
+            const uint32_t slot = (tail + __popc(bal & lt_mask)) & (kRing - 1);
+            qa[slot] = cur[j].x | (ka << 31);
+            qb[slot] = cur[j].y | (kb << 31);
+          }
+          tail += __popc(bal);
+          if (tail - head >= 32u) resolve(32u);
+        }
+      }
+      if (tail != head) resolve(tail - head);
+      __syncthreads();  // the bits and s_graph are rewritten next
+    }
+  }
+}
+
+// Phases 0 and 1, one cooperative launch: the offsets, then P[x] = x.
+__global__ void __launch_bounds__(512) k_batch_begin(BatchArgs a) {
+  unsigned int gen = 0;
+  if (blockIdx.x == 0) scan_tiles(a);
+  if (!grid_barrier(a.ctrl, gen, a.barrier_ns)) return;
   const uint64_t V = a.vtx_off[a.n_graphs];
   const uint64_t T = (uint64_t)gridDim.x * blockDim.x;
-  const uint64_t tid = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-  for (uint64_t x = tid; x < V; x += T) a.P[x] = (uint32_t)x;
-  if (!grid_barrier(c, gen, a.barrier_ns)) return;
+  for (uint64_t x = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; x < V; x += T) a.P[x] = (uint32_t)x;
+}
 
-  // 2. hooking over edge tiles, one warp per tile: lane 0 finds the tile's
-  // graph and broadcasts it, so no block barrier is taken per tile (a block
-  // would wait for its slowest warp's searches). Tile t goes to warp
-  // t % warps of block t / warps % gridDim.x: consecutive tiles, often of one
-  // graph, stay on one SM and share its L1.
+__device__ __forceinline__ bool aborted(const BatchArgs &a) { return *(volatile unsigned int *)&a.ctrl->abort != 0u; }
+
+// Phase 1. Bound by latency (52 of 64 cycles between a warp's instructions wait
+// for a load or a compare-and-swap), so 64 warps per SM at 32 registers: 2.03
+// ms on 2000 mixed graphs against 2.45 with 48 warps and 2.87 with 32. Several
+// edges per lane in lock step measured slower (2.3 to 2.5 ms), and so did
+// hooking every vertex under its smallest sampled neighbour first.
+template <int EPT, bool FILTER>
+__global__ void __launch_bounds__(512, 4) k_batch_hook(BatchArgs a) {
+  extern __shared__ uint32_t ring_smem[];
+  if (aborted(a)) return;
+  BatchCtrl *const c = a.ctrl;
+  // One warp per tile, so no block barrier is taken per tile (a block would
+  // wait for its slowest warp's searches). Tile t goes to warp t % warps of
+  // block t / warps % gridDim.x: consecutive tiles, often of one graph, stay
+  // on one SM and share its L1.
   uint32_t *const P = a.P;  // names are global ids: the slot of name x is P[x]
   WarpRing ring;
   if (FILTER) ring.init(ring_smem);
@@ -238,75 +488,91 @@ __global__ void __launch_bounds__(512) k_batched(BatchArgs a) {
   const uint64_t wid = (uint64_t)blockIdx.x * wpb + (threadIdx.x >> 5);  // block-major
   const uint64_t n_warps = wpb * gridDim.x;
   const uint64_t n_etiles = a.etile_off[a.n_graphs];
+  const uint32_t per_tile = c->tile_chunks;
   for (uint64_t t = wid; t < n_etiles; t += n_warps) {
-    uint64_t nv = 0, e0 = 0, e1 = 0, base64 = 0;
-    if (lane == 0) {
-      const uint32_t g = owner(a.etile_off, a.n_graphs, t);
-      e0 = a.edge_off[g] + (t - a.etile_off[g]) * a.tile_edges;
-      const uint64_t ge = a.edge_off[g + 1];
-      e1 = e0 + a.tile_edges < ge ? e0 + a.tile_edges : ge;
-      nv = a.vtx_off[g + 1] - a.vtx_off[g];
-      base64 = a.vtx_off[g];
-    }
-    nv = __shfl_sync(0xFFFFFFFFu, nv, 0);
-    e0 = __shfl_sync(0xFFFFFFFFu, e0, 0);
-    e1 = __shfl_sync(0xFFFFFFFFu, e1, 0);
-    const uint32_t base = (uint32_t)__shfl_sync(0xFFFFFFFFu, base64, 0);
-    for (uint64_t r0 = e0; r0 < e1; r0 += 32u * EPT) {
-      uint32_t u[EPT], v[EPT], pu[EPT], pv[EPT];
+    const uint32_t g = owner_warp(a.etile_off, a.n_graphs, t);
+    const uint64_t e0 = a.edge_off[g], n_e = a.edge_off[g + 1] - e0;
+    const uint64_t base64 = a.vtx_off[g], nv = a.vtx_off[g + 1] - base64;
+    const uint32_t base = (uint32_t)base64, stride = sample_stride(n_e, nv);
+    const uint64_t step = (uint64_t)stride * kChunkEdges;
+    uint64_t first = (t - a.etile_off[g]) * per_tile * step;
+    for (uint32_t k = 0; k < per_tile && first < n_e; ++k, first += step) {
+      const uint64_t last = first + kChunkEdges < n_e ? first + kChunkEdges : n_e;
+      for (uint64_t r0 = first; r0 < last; r0 += 32u * EPT) {
+        uint32_t u[EPT], v[EPT], pu[EPT], pv[EPT];
 #pragma unroll
-      for (int j = 0; j < EPT; ++j) {
-        const uint64_t i = r0 + (uint64_t)j * 32u + lane;
-        uint2 ed = make_uint2(0u, 0u);
-        bool ok = false;
-        if (i < e1) {
-          ed = ld_edge(a.edges + i);
-          ok = ed.x < nv && ed.y < nv;
-          if (!ok) atomicOr(&c->err, kErrRange);
+        for (int j = 0; j < EPT; ++j) {
+          const uint64_t i = r0 + (uint64_t)j * 32u + lane;
+          uint2 ed = make_uint2(0u, 0u);
+          bool ok = false;
+          if (i < last) {
+            ed = ld_edge(a.edges + e0 + i);
+            ok = ed.x < nv && ed.y < nv;
+            if (!ok) atomicOr(&c->err, kErrRange);
+          }
+          // an empty or invalid slot touches no memory: equal parents drop it
+          u[j] = ok ? base + ed.x : 0u;
+          v[j] = ok ? base + ed.y : 0u;
+          pu[j] = ok ? 1u : 0u;
+          pv[j] = pu[j];
         }
-        // an empty or invalid slot touches no memory: equal parents drop it
-        u[j] = ok ? base + ed.x : 0u;
-        v[j] = ok ? base + ed.y : 0u;
-        pu[j] = ok ? 1u : 0u;
-        pv[j] = pu[j];
-      }
 #pragma unroll
-      for (int j = 0; j < EPT; ++j) {
-        if (pu[j]) {
-          pu[j] = ldP(P + u[j]);
-          pv[j] = ldP(P + v[j]);
+        for (int j = 0; j < EPT; ++j) {
+          if (pu[j]) {
+            pu[j] = ldP(P + u[j]);
+            pv[j] = ldP(P + v[j]);
+          }
         }
-      }
 #pragma unroll
-      for (int j = 0; j < EPT; ++j) {
-        if (FILTER)
-          ring.push(P, pu[j] != pv[j], u[j], pu[j], v[j], pv[j]);
-        else
-          unite(P, u[j], pu[j], v[j], pv[j]);
+        for (int j = 0; j < EPT; ++j) {
+          if (FILTER)
+            ring.push(P, pu[j] != pv[j], u[j], pu[j], v[j], pv[j]);
+          else
+            unite(P, u[j], pu[j], v[j], pv[j]);
+        }
       }
     }
   }
   if (FILTER) ring.drain(P);
-  if (!grid_barrier(c, gen, a.barrier_ns)) return;
+}
 
-  // 3. compression: each vertex stores its root's name (read-only walks)
-  for (uint64_t x = tid; x < V; x += T) {
-    const uint32_t px = ldP_strong(P + x);
-    if (px == (uint32_t)x) continue;
-    uint32_t r = px, pr = ldP_strong(P + r);
-    while (pr != r) {
-      r = pr;
-      pr = ldP_strong(P + r);
+// Compression; kRefs: also each graph's reference, and nothing when no graph has a filtered phase.
+template <bool kRefs>
+__global__ void __launch_bounds__(256) k_batch_compress(BatchArgs a) {
+  if (aborted(a)) return;
+  uint32_t *const P = a.P;
+  const uint64_t T = (uint64_t)gridDim.x * blockDim.x, tid = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+  if (kRefs) {
+    if (a.chunk_off[a.n_graphs] == 0) return;
+    const uint32_t lane = threadIdx.x & 31u;
+    for (uint64_t g = tid / 32u; g < a.n_graphs; g += T / 32u) {
+      const uint64_t v0 = a.vtx_off[g], nv = a.vtx_off[g + 1] - v0;
+      if (sample_stride(a.edge_off[g + 1] - a.edge_off[g], nv) == 1u) continue;
+      const uint32_t r = walk_root(P, (uint32_t)(v0 + nv * lane / 32u));
+      const uint32_t votes = (uint32_t)__popc(__match_any_sync(0xFFFFFFFFu, r));
+      const uint32_t best = __reduce_max_sync(0xFFFFFFFFu, votes * 32u + lane) & 31u;
+      const uint32_t ref = __shfl_sync(0xFFFFFFFFu, r, (int)best);
+      if (lane == 0) a.ref[g] = ref;
     }
-    if (r != px) stP(P + x, r);
   }
-  if (!grid_barrier(c, gen, a.barrier_ns)) return;
+  compress(P, a.vtx_off[a.n_graphs], tid, T);
+}
 
-  // 4. graph-local labels, in place
+__global__ void __launch_bounds__(512, 3) k_batch_filtered(BatchArgs a) {
+  extern __shared__ uint32_t ring_smem[];  // the bits, then the queues
+  if (aborted(a)) return;
+  filtered_phase(a, ring_smem, ring_smem + kBitsMax / 32u);
+}
+
+// Graph-local labels, in place.
+__global__ void __launch_bounds__(512) k_batch_labels(BatchArgs a) {
+  __shared__ uint64_t s_tile[4];
+  if (aborted(a)) return;
+  uint32_t *const P = a.P;
   const uint64_t n_vtiles = a.vtile_off[a.n_graphs];
   for (uint64_t t = blockIdx.x; t < n_vtiles; t += gridDim.x) {
-    if (threadIdx.x == 0) {
-      const uint32_t g = owner(a.vtile_off, a.n_graphs, t);
+    if (threadIdx.x < 32) {
+      const uint32_t g = owner_warp(a.vtile_off, a.n_graphs, t);
       const uint64_t x0 = a.vtx_off[g] + (t - a.vtile_off[g]) * a.tile_vertices;
       const uint64_t x1 = a.vtx_off[g + 1];
       s_tile[1] = x0;
@@ -319,18 +585,10 @@ __global__ void __launch_bounds__(512) k_batched(BatchArgs a) {
     __syncthreads();
     for (uint64_t x = x0 + threadIdx.x; x < x1; x += blockDim.x) P[x] = ldP_strong(P + x) - base;
   }
-  CC_BATCH_TICK(5);
 }
 
 }  // namespace
 }  // namespace cc
-
-#ifdef CC_BATCH_CLOCK
-// Diagnostics builds only: the timer readings of the last batched run.
-extern "C" __attribute__((visibility("default"))) int cc_batch_clock_read(unsigned long long out[8]) {
-  return (int)cudaMemcpyFromSymbol(out, cc::g_batch_clock, 8 * sizeof(unsigned long long));
-}
-#endif
 
 using cc::BatchArgs;
 using cc::BatchCtrl;
@@ -341,7 +599,7 @@ struct cc_batch {
   cc_batch_config cfg{};
   BatchCtrl *ctrl = nullptr;
   BatchCtrl *host_ctrl = nullptr;
-  uint64_t *tile_off = nullptr;  // 2 * (max_graphs + 1)
+  uint64_t *tile_off = nullptr;  // 3 * (max_graphs + 1), then max_graphs references (uint32)
   cudaStream_t last = nullptr;
   // the last cc_batch_tune: every candidate with its best time
   cc_batch_config tuned[64];
@@ -375,29 +633,47 @@ cc_batch_config default_cfg() {
 }
 
 template <int EPT, bool FILTER>
-cudaError_t launch_batched_t(const cc_batch_config &cfg, BatchArgs &a, cudaStream_t s) {
-  const void *k = (const void *)cc::k_batched<EPT, FILTER>;
+cudaError_t launch_hook(const cc_batch_config &cfg, const BatchArgs &a, cudaStream_t s) {
   const size_t smem = FILTER ? (size_t)(cfg.block_size / 32) * 4 * cc::kRing * sizeof(uint32_t) : 0;
-  int occ = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, cfg.block_size, smem);
-  if (e != cudaSuccess) return e;
-  if (occ < 1) return cudaErrorInvalidConfiguration;
-  const unsigned grid = (unsigned)(cc::num_sms() * occ);
-  void *args[] = {&a};
-  e = cudaLaunchCooperativeKernel(k, dim3(grid), dim3(cfg.block_size), args, smem, s);
+  const unsigned grid = (unsigned)cc::persistent_cap((const void *)cc::k_batch_hook<EPT, FILTER>, cfg.block_size, smem);
+  cc::k_batch_hook<EPT, FILTER><<<grid, cfg.block_size, smem, s>>>(a);
   cc::note_launch();
-  return e;
+  return cudaGetLastError();
 }
 
 cudaError_t launch_batched(const cc_batch_config &cfg, BatchArgs &a, cudaStream_t s) {
-  switch (cfg.edges_per_thread * 2 + cfg.filter) {
-    case 2: return launch_batched_t<1, false>(cfg, a, s);
-    case 3: return launch_batched_t<1, true>(cfg, a, s);
-    case 4: return launch_batched_t<2, false>(cfg, a, s);
-    case 5: return launch_batched_t<2, true>(cfg, a, s);
-    case 8: return launch_batched_t<4, false>(cfg, a, s);
-    default: return launch_batched_t<4, true>(cfg, a, s);
+  cudaError_t e;
+  {
+    const void *k = (const void *)cc::k_batch_begin;
+    const unsigned grid = (unsigned)cc::persistent_cap(k, 512, 0);
+    void *args[] = {&a};
+    if ((e = cudaLaunchCooperativeKernel(k, dim3(grid), dim3(512), args, 0, s)) != cudaSuccess) return e;
+    cc::note_launch();
   }
+  const unsigned gc = (unsigned)cc::persistent_cap((const void *)cc::k_batch_compress<true>, 256, 0);
+  switch (cfg.edges_per_thread * 2 + cfg.filter) {
+    case 2: e = launch_hook<1, false>(cfg, a, s); break;
+    case 3: e = launch_hook<1, true>(cfg, a, s); break;
+    case 4: e = launch_hook<2, false>(cfg, a, s); break;
+    case 5: e = launch_hook<2, true>(cfg, a, s); break;
+    case 8: e = launch_hook<4, false>(cfg, a, s); break;
+    default: e = launch_hook<4, true>(cfg, a, s); break;
+  }
+  if (e != cudaSuccess) return e;
+  cc::k_batch_compress<true><<<gc, 256, 0, s>>>(a);
+  cc::note_launch();
+  const size_t smem = cc::kBitsMax / 8 + (size_t)(512 / 32) * 2 * cc::kRing * sizeof(uint32_t);
+  static std::atomic<unsigned long long> smem_set{0};
+  const void *kf = (const void *)cc::k_batch_filtered;
+  if ((e = cc::ensure_func_attr(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem, smem_set)) != cudaSuccess) return e;
+  cc::k_batch_filtered<<<(unsigned)cc::persistent_cap(kf, 512, smem), 512, smem, s>>>(a);
+  cc::note_launch();
+  cc::k_batch_compress<false><<<gc, 256, 0, s>>>(a);
+  cc::note_launch();
+  const unsigned gl = (unsigned)cc::persistent_cap((const void *)cc::k_batch_labels, 512, 0);
+  cc::k_batch_labels<<<gl, 512, 0, s>>>(a);
+  cc::note_launch();
+  return cudaGetLastError();
 }
 
 cc_status from_cuda(cudaError_t e) {
@@ -423,6 +699,7 @@ struct DeviceGuard {
 cc_status enqueue(cc_batch *b, const cc_batch_config &cfg, uint32_t n_graphs, const uint64_t *vtx_off,
                   const uint64_t *edge_off, const uint32_t *edges, uint32_t *L, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(b->ctrl, 0, 3 * sizeof(unsigned int), s);  // barrier state and abort
+  if (e == cudaSuccess) e = cudaMemsetAsync(&b->ctrl->segs, 0, sizeof(unsigned long long), s);
   if (e != cudaSuccess) return from_cuda(e);
   BatchArgs a;
   a.n_graphs = n_graphs;
@@ -431,9 +708,12 @@ cc_status enqueue(cc_batch *b, const cc_batch_config &cfg, uint32_t n_graphs, co
   a.edges = reinterpret_cast<const uint2 *>(edges);
   a.P = L;
   a.etile_off = b->tile_off;
-  a.vtile_off = b->tile_off + (b->max_graphs + 1);
+  a.vtile_off = a.etile_off + (b->max_graphs + 1);
+  a.chunk_off = a.vtile_off + (b->max_graphs + 1);
+  a.ref = reinterpret_cast<uint32_t *>(a.chunk_off + (b->max_graphs + 1));
   a.tile_edges = cfg.tile_edges;
   a.tile_vertices = cfg.tile_vertices;
+  a.hook_warps = (uint32_t)(cc::num_sms() * 64);
   a.barrier_ns = cfg.barrier_wait_us ? (unsigned long long)cfg.barrier_wait_us * 1000ULL : cc::kBarrierTimeoutNs;
   a.ctrl = b->ctrl;
   return from_cuda(launch_batched(cfg, a, s));
@@ -465,7 +745,7 @@ cc_status cc_batch_create(uint32_t max_graphs, cc_batch **out) {
   cudaError_t e = cudaGetDevice(&b->device);
   if (e == cudaSuccess) e = cudaMalloc((void **)&b->ctrl, sizeof(BatchCtrl));
   if (e == cudaSuccess) e = cudaMallocHost((void **)&b->host_ctrl, sizeof(BatchCtrl));
-  if (e == cudaSuccess) e = cudaMalloc((void **)&b->tile_off, 2 * ((size_t)max_graphs + 1) * sizeof(uint64_t));
+  if (e == cudaSuccess) e = cudaMalloc((void **)&b->tile_off, 3 * ((size_t)max_graphs + 1) * sizeof(uint64_t) + (size_t)max_graphs * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMemset(b->ctrl, 0, sizeof(BatchCtrl));
   if (e != cudaSuccess) {
     cc_batch_destroy(b);

@@ -81,6 +81,13 @@ __device__ __forceinline__ uint2 ld_edge(const uint2 *a) {
   return r;
 }
 
+// The same, kept where it stands in the program (see ld_edges_now).
+__device__ __forceinline__ uint2 ld_edge_now(const uint2 *a) {
+  uint2 r;
+  asm volatile("ld.global.nc.L1::no_allocate.v2.u32 {%0,%1}, [%2];" : "=r"(r.x), "=r"(r.y) : "l"(a));
+  return r;
+}
+
 // Parent-array load. A weak load may be served from this SM's L1 and so be
 // stale; by the facts above a stale value is an older ancestor, which keeps
 // every search correct. (CAS results always come from L2.)
