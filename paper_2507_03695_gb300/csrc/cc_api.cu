@@ -49,6 +49,7 @@ struct cc_graph {
   uint32_t *cand_list = nullptr;  // listed candidates of the root selection (cand_cap entries), f = R only
   uint32_t cand_cap = 0;
   cc::WideHot *wide_hot = nullptr;  // wide hot-vertex table, or null
+  uint32_t *bits = nullptr;         // vertex bits of the edge pass on small graphs, or null
   uint32_t *z = nullptr;   // zero-tree bitmap (one bit per name), or null
   size_t z_bytes = 0;
   bool z_forced = false;   // CC_FILTER_BITMAP: always used
@@ -85,6 +86,12 @@ bool wants_wide_hot(const cc_options &o, uint64_t n) {
   return o.mode == CC_ROOT_MAXDEG && o.root_hint == CC_ROOT_AUTO && o.root_select != CC_ROOT_SELECT_SAMPLED &&
          o.filter != CC_FILTER_OFF && o.filter != CC_FILTER_BITMAP && o.block_size == 0 && o.edges_per_thread == 0 &&
          cc::wide_hot_fits(n);
+}
+
+// The vertex bits of small graphs: the edge pass's default shape.
+bool wants_bits(const cc_options &o, uint64_t n) {
+  return n >= 1 && n <= cc::kBitsVertices && o.filter != CC_FILTER_OFF && o.filter != CC_FILTER_BITMAP &&
+         o.block_size == 0 && o.edges_per_thread == 0 && o.initial_push != CC_PUSH_ON;
 }
 
 struct DeviceGuard {
@@ -138,18 +145,40 @@ int eff_filter(const cc_graph *g) {
 int eff_ept(const cc_graph *g) { return g->opt.edges_per_thread ? g->opt.edges_per_thread : 4; }
 int eff_block(const cc_graph *g) { return g->opt.block_size ? g->opt.block_size : 512; }
 
+void dev_free(cc_graph *g, void *p, size_t bytes) {
+  if (p) {
+    cudaFree(p);
+    g->owned -= bytes;
+  }
+}
+
+// Scratch that only speeds a run up: the passes that use it fall back to the
+// general ones without it.
+void free_optional(cc_graph *g) {
+  dev_free(g, g->wide_hot, sizeof(cc::WideHot));
+  dev_free(g, g->bits, cc::bits_bytes(g->n));
+  g->wide_hot = nullptr;
+  g->bits = nullptr;
+}
+
+// Within the budget; a needed buffer displaces the optional ones.
 cudaError_t dev_alloc(cc_graph *g, void **p, size_t bytes) {
-  if (g->opt.hbm_budget_bytes && g->owned + bytes > g->opt.hbm_budget_bytes)
-    return cudaErrorMemoryAllocation;
+  const uint64_t budget = g->opt.hbm_budget_bytes;
+  if (budget && g->owned + bytes > budget) free_optional(g);
+  if (budget && g->owned + bytes > budget) return cudaErrorMemoryAllocation;
   cudaError_t e = cudaMalloc(p, bytes ? bytes : 16);
   if (e == cudaSuccess) g->owned += bytes;
   return e;
 }
 
-void dev_free(cc_graph *g, void *p, size_t bytes) {
-  if (p) {
-    cudaFree(p);
-    g->owned -= bytes;
+void optional_alloc(cc_graph *g, void **p, size_t bytes) {
+  const uint64_t budget = g->opt.hbm_budget_bytes;
+  if (budget && g->owned + bytes > budget) return;
+  if (cudaMalloc(p, bytes) == cudaSuccess) {
+    g->owned += bytes;
+  } else {
+    *p = nullptr;
+    cudaGetLastError();  // not an error of the call
   }
 }
 
@@ -291,8 +320,7 @@ cc_status cc_create(uint64_t n_vertices, uint64_t n_edges_capacity, const cc_opt
   const bool rf = o.mode == CC_ROOT_MAXDEG;
   const size_t need = p_bytes(n_vertices) +
                       (rf ? (size_t)n_vertices * 4 + sizeof(cc::CertScratch) + (size_t)cc::cand_list_cap(n_vertices) * 4
-                          : 0) + sizeof(Ctrl) + (wants_wide_hot(o, n_vertices) ? sizeof(cc::WideHot) : 0) +
-                      (size_t)n_edges_capacity * 8 + (wants_z(o, n_vertices) ? z_bytes_for(n_vertices) : 0) +
+                          : 0) + sizeof(Ctrl) + (size_t)n_edges_capacity * 8 + (wants_z(o, n_vertices) ? z_bytes_for(n_vertices) : 0) +
                       (wants_push(o) ? (size_t)push_cap_for(n_vertices) * 4 : 0);
   if (o.hbm_budget_bytes && need > o.hbm_budget_bytes) return CC_ERR_OOM;
 
@@ -324,9 +352,6 @@ cc_status cc_create(uint64_t n_vertices, uint64_t n_edges_capacity, const cc_opt
       if ((e = dev_alloc(g, (void **)&g->cert, sizeof(cc::CertScratch))) != cudaSuccess) break;
       g->cand_cap = cc::cand_list_cap(n_vertices);
       if ((e = dev_alloc(g, (void **)&g->cand_list, (size_t)g->cand_cap * 4)) != cudaSuccess) break;
-      if (wants_wide_hot(o, n_vertices) &&
-          (e = dev_alloc(g, (void **)&g->wide_hot, sizeof(cc::WideHot))) != cudaSuccess)
-        break;
     }
     if (n_edges_capacity) {
       if ((e = dev_alloc(g, (void **)&g->staging, (size_t)n_edges_capacity * 8)) != cudaSuccess) break;
@@ -342,6 +367,8 @@ cc_status cc_create(uint64_t n_vertices, uint64_t n_edges_capacity, const cc_opt
       g->z_forced = o.filter == CC_FILTER_BITMAP;
       if ((e = cudaMemset(g->z, 0, g->z_bytes)) != cudaSuccess) break;
     }
+    if (wants_wide_hot(o, n_vertices)) optional_alloc(g, (void **)&g->wide_hot, sizeof(cc::WideHot));
+    if (wants_bits(o, n_vertices)) optional_alloc(g, (void **)&g->bits, cc::bits_bytes(n_vertices));
     if ((e = cudaStreamCreateWithFlags(&g->copy_stream, cudaStreamNonBlocking)) != cudaSuccess) break;
     if ((e = cudaEventCreateWithFlags(&g->copy_ev, cudaEventDisableTiming)) != cudaSuccess) break;
     if ((e = cudaMemset(g->ctrl, 0, sizeof(Ctrl))) != cudaSuccess) break;
@@ -371,7 +398,7 @@ void cc_destroy(cc_graph *g) {
   dev_free(g, g->cnt, g->cnt_bytes);
   dev_free(g, g->cert, sizeof(cc::CertScratch));
   dev_free(g, g->cand_list, (size_t)g->cand_cap * 4);
-  dev_free(g, g->wide_hot, sizeof(cc::WideHot));
+  free_optional(g);
   dev_free(g, g->ctrl, sizeof(Ctrl));
   dev_free(g, g->staging, (size_t)g->capacity * 8);
   dev_free(g, g->label_dev, (size_t)g->n * 4);
@@ -425,9 +452,13 @@ cc_status cc_run(cc_graph *g, const uint32_t *edges_dev, uint64_t n_edges, uint3
   uint32_t *Z = (g->z && (g->z_forced || exact)) ? g->z : nullptr;
   const uint32_t *zsel = (Z && !g->z_forced) ? &g->ctrl->cert : nullptr;
   record(g, 2, s);
-  CC_TRY(cc::launch_edge_pass(g->rf, eff_filter(g), eff_ept(g), eff_block(g), span, g->P, n, g->ctrl,
-                              nullptr, s, Z, zsel, false, nullptr, exact ? &g->ctrl->cert : nullptr, true,
-                              exact ? g->cert->hot : nullptr, exact ? g->wide_hot : nullptr));
+  if (g->bits && cc::bits_pass_fits(n, n_edges)) {
+    CC_TRY(cc::launch_edge_pass_bits(g->rf, span, g->P, n, g->ctrl, g->bits, s));
+  } else {
+    CC_TRY(cc::launch_edge_pass(g->rf, eff_filter(g), eff_ept(g), eff_block(g), span, g->P, n, g->ctrl,
+                                nullptr, s, Z, zsel, false, nullptr, exact ? &g->ctrl->cert : nullptr, true,
+                                exact ? g->cert->hot : nullptr, exact ? g->wide_hot : nullptr));
+  }
   record(g, 3, s);
   CC_TRY(cc::launch_flatten(g->rf, g->opt.label_space, g->P, n, L_out_dev, g->ctrl, s));
   record(g, 4, s);

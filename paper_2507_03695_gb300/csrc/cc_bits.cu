@@ -1,0 +1,314 @@
+// cc_bits.cu - the edge pass on graphs whose vertices fit, a bit each, in one
+// block's shared memory (at most kBitsVertices) and that have at least
+// kBitsMinDegree edges per vertex.
+//
+// The general pass is slow there for two reasons. It looks up both endpoints
+// of every edge in L2, although after a small part of the edges nearly all of
+// them lie inside the giant component. And that small part takes most of the
+// time: all searches meet on the few roots of the growing trees, and loads and
+// compare-and-swaps of one L2 sector are served one after another (R-MAT
+// scale 16 under f = id: 1.0M of its 1.05M edges in flight at once take 0.55
+// ms, and the general pass throttles itself to 512 warps to reach 0.09). So:
+//   1. linking rounds. Each takes a sample of the edges and lowers the parent
+//      of the larger of the two endpoints' roots to the smaller one, by a
+//      reduction that nothing waits for; the lanes of a warp that lower one
+//      root do it once. A link that another one overwrites is lost, which is
+//      harmless: step 3 goes through every edge. After each round all vertices
+//      are compressed to their roots. The samples shrink fourfold per round
+//      while the trees grow more than that, so a root gets enough edges to be
+//      linked and too few to queue up behind.
+//   2. the last compression also writes one bit per vertex: whether it is in
+//      the reference tree, the one that most of 32 sampled endpoints are in.
+//   3. every block copies the bits into its shared memory and streams the
+//      edges: one whose endpoints are both marked is inside the reference tree
+//      for good, and costs two shared-memory loads. The others are queued and
+//      joined exactly as in the general pass.
+// Measured, edge pass in microseconds, general pass and this one: R-MAT scale
+// 16 (f = id) 101 -> 66, scale 20 (16M edges) 269 -> 150; uniform graphs of
+// 2^18 vertices with four edges per vertex 149 -> 76, of 2^20 with ten 308 ->
+// 135. What bounds it now: at scale 16 the launches (ten of 2 to 4 us, the
+// first sample's and step 3's loads aside), at scale 20 step 3 (73 us for 128
+// MB of edges: a tenth of them still leads to a search).
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "cc_device.cuh"
+#include "cc_internal.h"
+
+namespace cc {
+
+namespace {
+
+constexpr uint32_t kChunkQuads = 64;  // 128 edges, four per lane of a warp
+constexpr int kFilterBlock = 1024;
+constexpr int kLinkBlock = 256;
+constexpr size_t kFilterQueueBytes = (kFilterBlock / 32) * 2 * kRing * sizeof(uint32_t);
+static_assert(kBitsVertices / 8 + kFilterQueueBytes <= 224 * 1024, "the bits and the queues fit a block's shared memory");
+
+// One linking round over the chunks k * stride + first. kFirst: P holds every
+// vertex's own name, so the endpoints need no parent loads.
+template <class F, bool kFirst>
+__global__ void __launch_bounds__(kLinkBlock) k_bits_link(const uint4 *__restrict__ e4, uint64_t n_quads,
+                                                          uint32_t stride, uint32_t first, uint32_t *P, uint32_t n,
+                                                          const Ctrl *ctrl) {
+  const F fn = F::load(ctrl);
+  uint32_t *const S = slots<F>(P);
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint64_t step = (uint64_t)stride * kChunkQuads;
+  const uint64_t hop = (uint64_t)gridDim.x * (kLinkBlock / 32) * step;
+  for (uint64_t q0 = ((uint64_t)blockIdx.x * (kLinkBlock / 32) + (threadIdx.x >> 5)) * step + first * kChunkQuads;
+       q0 < n_quads; q0 += hop) {
+    uint32_t x[8], p[8];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const uint64_t q = q0 + 32u * j + lane;
+      uint4 e = make_uint4(0u, 0u, 0u, 0u);
+      if (q < n_quads) e = __ldg(e4 + q);
+      if (max(max(e.x, e.y), max(e.z, e.w)) >= n) e = make_uint4(0u, 0u, 0u, 0u);  // reported by the filter
+      x[4 * j] = e.x;
+      x[4 * j + 1] = e.y;
+      x[4 * j + 2] = e.z;
+      x[4 * j + 3] = e.w;
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) p[i] = kFirst ? fn.f(x[i]) : ldP(P + x[i]);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const uint32_t a = p[2 * k], b = p[2 * k + 1], hi = max(a, b), lo = min(a, b);
+      if (kFirst) {  // the targets are mostly distinct
+        if (hi != lo) atomicMin(S + hi, lo);
+      } else {
+        const uint32_t act = __ballot_sync(0xFFFFFFFFu, hi != lo);
+        if (hi != lo) {
+          const uint32_t peers = __match_any_sync(act, hi);
+          const uint32_t least = __reduce_min_sync(peers, lo);
+          if ((peers & ((1u << lane) - 1u)) == 0u) atomicMin(S + hi, least);
+        }
+      }
+    }
+  }
+}
+
+// Compression, four vertices per thread. Short walks only read, so that every
+// vertex ends at its root (a split stored late would put an older ancestor
+// back, and a vertex that does not name its root spoils the next round:
+// uniform graphs then reached step 3 in many trees, 415 us instead of 117), and
+// read through L1, which answers the many loads of one root. A chain of links
+// can be as long as the graph (a path whose ids ascend): after kShortWalk
+// steps a walk splits its path and reads past L1, to gain from the others'
+// splitting. kBits: also the reference and the bits (32 per word, the words
+// of a warp step's 128 vertices together; bits from n on are 0).
+constexpr int kShortWalk = 16;
+
+template <class F, bool kBits>
+__global__ void __launch_bounds__(256) k_bits_build(const uint4 *__restrict__ e4, uint64_t n_quads, uint32_t *P,
+                                                    uint32_t n, Ctrl *ctrl, uint32_t *bits) {
+  __shared__ uint32_t s_ref;
+  const F fn = F::load(ctrl);
+  uint32_t *const S = slots<F>(P);
+  const uint32_t lane = threadIdx.x & 31u;
+  if (kBits && threadIdx.x < 32) {
+    // compression moves no vertex to another root, so every block finds the
+    // same reference whatever the others have done already
+    uint32_t x = __ldg(e4 + n_quads * lane / 32u).x;
+    if (x >= n) x = 0u;
+    const uint32_t r = root_name(S, fn.f(x), ldP(P + x));
+    const uint32_t votes = (uint32_t)__popc(__match_any_sync(0xFFFFFFFFu, r));
+    const uint32_t best = __reduce_max_sync(0xFFFFFFFFu, votes * 32u + lane) & 31u;
+    const uint32_t ref = __shfl_sync(0xFFFFFFFFu, r, (int)best);
+    if (lane == 0) {
+      s_ref = ref;
+      if (blockIdx.x == 0) ctrl->ref = ref;
+    }
+  }
+  if (kBits) __syncthreads();
+  const uint32_t ref = kBits ? s_ref : 0u;
+  const uint32_t groups = (n + 127u) / 128u;  // of 128 vertices, one per warp step
+  for (uint32_t g = blockIdx.x * 8u + (threadIdx.x >> 5); g < groups; g += gridDim.x * 8u) {
+    const uint32_t v = g * 128u + 4u * lane;
+    uint32_t nib = 0;
+    if (v < n) {  // P is padded to a multiple of four entries
+      uint32_t p0[4], c[4], r[4], run = 0;
+      asm volatile("ld.global.v4.u32 {%0,%1,%2,%3}, [%4];"
+                   : "=r"(p0[0]), "=r"(p0[1]), "=r"(p0[2]), "=r"(p0[3])
+                   : "l"(P + v)
+                   : "memory");
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        c[k] = fn.f(v + k);
+        r[k] = p0[k];
+        run |= (uint32_t)(v + k < n && r[k] != c[k] && r[k] != 0u) << k;
+      }
+      for (int steps = 0; run; ++steps) {
+        uint32_t w[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if ((run >> k) & 1u) w[k] = steps < kShortWalk ? ldP(S + r[k]) : ldP_cg(S + r[k]);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if ((run >> k) & 1u) {
+            if (w[k] != r[k] && steps >= kShortWalk) stP(S + c[k], w[k]);  // the parent is not a root: split past it
+            if (w[k] == r[k] || w[k] == 0u) run &= ~(1u << k);
+            c[k] = r[k];
+            r[k] = w[k];
+          }
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (v + k >= n) continue;
+        if (r[k] != p0[k]) stP(P + v + k, r[k]);
+        nib |= (uint32_t)(r[k] == ref) << k;
+      }
+    }
+    if (kBits) {
+      const uint32_t word = __reduce_or_sync(0xFFu << (lane & 24u), nib << (4u * (lane & 7u)));
+      if ((lane & 7u) == 0u) bits[g * 4u + (lane >> 3)] = word;
+    }
+  }
+}
+
+// Step 3. One block of 32 warps per SM; a warp's next chunk is loaded while it
+// works on one.
+template <class F>
+__global__ void __launch_bounds__(kFilterBlock, 1)
+    k_bits_filter(const uint4 *__restrict__ e4, uint64_t n_quads, const uint2 *head, const uint2 *tail, uint32_t *P,
+                  uint32_t n, Ctrl *ctrl, const uint32_t *__restrict__ all_bits) {
+  extern __shared__ uint32_t smem[];
+  const F fn = F::load(ctrl);
+  uint32_t *const S = slots<F>(P);
+  const uint32_t ref = ld_volatile_u32(&ctrl->ref);
+  const uint32_t groups = (n + 127u) / 128u;
+  uint32_t *const bits = smem;
+  for (uint32_t i = threadIdx.x; i < groups; i += kFilterBlock)
+    reinterpret_cast<uint4 *>(bits)[i] = __ldg(reinterpret_cast<const uint4 *>(all_bits) + i);
+  const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5, lt_mask = (1u << lane) - 1u;
+  // a queue of ids per warp (top bit: marked), as deep as the warp ring's
+  uint32_t *const qa = smem + 4u * groups + wid * 2 * kRing, *const qb = qa + kRing;
+  uint32_t q_head = 0, q_tail = 0;
+  __syncthreads();
+  const uint64_t t = blockIdx.x * (uint64_t)kFilterBlock + threadIdx.x;
+  if (t == 0 && head) single_edge<F, true>(P, fn, head, n, ctrl);
+  if (t == 1 && tail) single_edge<F, true>(P, fn, tail, n, ctrl);
+  auto resolve = [&](uint32_t count) {
+    __syncwarp();
+    const uint32_t slot = (q_head + lane) & (kRing - 1);
+    const uint32_t xa = qa[slot], xb = qb[slot];
+    __syncwarp();
+    if (lane < count) {
+      const bool ka = xa >> 31, kb = xb >> 31;
+      const uint32_t va = xa & 0x7FFFFFFFu, vb = xb & 0x7FFFFFFFu;
+      uint32_t pa = ref, pb = ref;  // a marked vertex's parent was the reference
+      if (!ka) pa = ldP_cg(P + va);
+      if (!kb) pb = ldP_cg(P + vb);
+      if (!ka && pa == ref) atomicOr(bits + (va >> 5), 1u << (va & 31u));
+      if (!kb && pb == ref) atomicOr(bits + (vb >> 5), 1u << (vb & 31u));
+      if (pa != pb) unite<true>(S, fn.f(va), pa, fn.f(vb), pb);
+    }
+    q_head += count;
+  };
+  const uint64_t pol = policy_evict_first();
+  const uint64_t chunks = (n_quads + kChunkQuads - 1) / kChunkQuads, full = n_quads / kChunkQuads;
+  const uint64_t hop = (uint64_t)gridDim.x * (kFilterBlock / 32);
+  uint64_t ch = (uint64_t)wid * gridDim.x + blockIdx.x;
+  uint4 e[2];
+  auto load = [&]() {
+    const uint4 *const p = e4 + ch * kChunkQuads + lane;
+    if (ch < full) {
+      e[0] = ld_edges_now(p, pol);
+      e[1] = ld_edges_now(p + 32, pol);
+    } else {
+      const uint32_t left = (uint32_t)(n_quads - ch * kChunkQuads);
+      e[0] = lane < left ? ld_edges_now(p, pol) : make_uint4(0u, 0u, 0u, 0u);
+      e[1] = lane + 32u < left ? ld_edges_now(p + 32, pol) : make_uint4(0u, 0u, 0u, 0u);
+    }
+  };
+  if (ch < chunks) load();
+  while (ch < chunks) {
+    uint32_t x[8] = {e[0].x, e[0].y, e[0].z, e[0].w, e[1].x, e[1].y, e[1].z, e[1].w};
+    ch += hop;
+    if (ch < chunks) load();
+    const uint32_t top = max(max(max(x[0], x[1]), max(x[2], x[3])), max(max(x[4], x[5]), max(x[6], x[7])));
+    if (top >= n) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) guard(x[2 * k], x[2 * k + 1], n, ctrl);
+    }
+    uint32_t w[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[i] = bits[x[i] >> 5];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const uint32_t xa = x[2 * k], xb = x[2 * k + 1];
+      // the vertex's bit comes to the bottom (the rotation takes the count modulo 32)
+      const uint32_t ka = __funnelshift_r(w[2 * k], w[2 * k], xa), kb = __funnelshift_r(w[2 * k + 1], w[2 * k + 1], xb);
+      const bool keep = !(ka & kb & 1u);
+      const uint32_t bal = __ballot_sync(0xFFFFFFFFu, keep);
+      if (!bal) continue;
+      if (keep) {
+        const uint32_t slot = (q_tail + __popc(bal & lt_mask)) & (kRing - 1);
+        qa[slot] = xa | (ka << 31);
+        qb[slot] = xb | (kb << 31);
+      }
+      q_tail += __popc(bal);
+      if (q_tail - q_head >= 32u) resolve(32u);
+    }
+  }
+  if (q_tail != q_head) resolve(q_tail - q_head);
+}
+
+// Linking rounds and their samples: two edges per vertex in the first round, a
+// quarter of that in each of the next. Edge pass in microseconds on uniform
+// graphs of 2^20 vertices with 3 / 10 edges per vertex and R-MAT scales 16 and
+// 18 under f = id: 117 / 135 / 66 / 75. With one edge per vertex 380 / 956 /
+// 70 / 99 and with three rounds 302 / 662 / 57 / 64, because step 3 then meets
+// many trees; with three edges per vertex 118 / 135 / 65 / 104.
+constexpr int kRounds = 4;
+constexpr uint64_t kFirstSample = 2, kShrink = 4;
+constexpr uint64_t kMinSampleChunks = 32;
+
+template <class F>
+cudaError_t bits_pass(const EdgeSpan &e, uint32_t *P, uint32_t n, Ctrl *ctrl, uint32_t *bits, cudaStream_t s) {
+  const uint64_t chunks = (e.n_quads + kChunkQuads - 1) / kChunkQuads;
+  const unsigned gb = clamp_grid(((uint64_t)n + 1023) / 1024, persistent_cap((const void *)k_bits_build<F, true>, 256, 0));
+  uint64_t sample = kFirstSample * n / (2 * kChunkQuads) + 1;  // in chunks
+  for (int r = 0; r < kRounds; ++r, sample = sample / kShrink > kMinSampleChunks ? sample / kShrink : kMinSampleChunks) {
+    const uint64_t stride = chunks > sample ? chunks / sample : 1;
+    const uint32_t first = (uint32_t)((uint64_t)r % stride);  // other edges than the round before
+    const uint64_t taken = (chunks + stride - 1) / stride;
+    const void *k = r ? (const void *)k_bits_link<F, false> : (const void *)k_bits_link<F, true>;
+    const unsigned gl = clamp_grid((taken + kLinkBlock / 32 - 1) / (kLinkBlock / 32), persistent_cap(k, kLinkBlock, 0));
+    if (r == 0)
+      k_bits_link<F, true><<<gl, kLinkBlock, 0, s>>>(e.quads, e.n_quads, (uint32_t)stride, first, P, n, ctrl);
+    else
+      k_bits_link<F, false><<<gl, kLinkBlock, 0, s>>>(e.quads, e.n_quads, (uint32_t)stride, first, P, n, ctrl);
+    note_launch();
+    if (r + 1 < kRounds)
+      k_bits_build<F, false><<<gb, 256, 0, s>>>(e.quads, e.n_quads, P, n, ctrl, nullptr);
+    else
+      k_bits_build<F, true><<<gb, 256, 0, s>>>(e.quads, e.n_quads, P, n, ctrl, bits);
+    note_launch();
+  }
+  const void *k = (const void *)k_bits_filter<F>;
+  static std::atomic<unsigned long long> smem_set{0};
+  const cudaError_t err = ensure_func_attr(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)(kBitsVertices / 8 + kFilterQueueBytes), smem_set);
+  if (err != cudaSuccess) return err;
+  const unsigned gf = clamp_grid((chunks + kFilterBlock / 32 - 1) / (kFilterBlock / 32), (uint64_t)num_sms());
+  k_bits_filter<F><<<gf, kFilterBlock, bits_bytes(n) + kFilterQueueBytes, s>>>(e.quads, e.n_quads, e.head, e.tail, P, n,
+                                                                             ctrl, bits);
+  note_launch();
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+bool bits_pass_fits(uint64_t n_vertices, uint64_t n_edges) {
+  return n_vertices >= 1 && n_vertices <= kBitsVertices && n_edges >= kBitsMinEdges && n_edges < kBitsMaxEdges &&
+         n_edges >= kBitsMinDegree * n_vertices;
+}
+
+cudaError_t launch_edge_pass_bits(bool rf, const EdgeSpan &e, uint32_t *P, uint32_t n, Ctrl *ctrl, uint32_t *bits,
+                                  cudaStream_t s) {
+  return rf ? bits_pass<RootR>(e, P, n, ctrl, bits, s) : bits_pass<RootId>(e, P, n, ctrl, bits, s);
+}
+
+}  // namespace cc

@@ -307,6 +307,26 @@ __device__ __forceinline__ void log_hooks_warp(uint32_t *log, uint32_t hooked, u
   if (hooked != kNoHook) log[1u + base + (uint32_t)__popc(bal & lt_mask)] = hooked;
 }
 
+// Range check of one edge; an out-of-range id flags the error and turns the
+// edge into the no-op self-loop (0, 0).
+__device__ __forceinline__ void guard(uint32_t &a, uint32_t &b, uint32_t n, Ctrl *ctrl) {
+  if (a >= n || b >= n) {
+    set_err(ctrl, kErrRange);
+    a = 0u;
+    b = 0u;
+  }
+}
+
+template <class F, bool kCG = false>
+__device__ __forceinline__ void single_edge(uint32_t *P, const F fn, const uint2 *e, uint32_t n,
+                                            Ctrl *ctrl, uint32_t *log = nullptr) {
+  uint2 x = ld_edge(e);
+  guard(x.x, x.y, n, ctrl);
+  const UniteResult r =
+      unite<kCG>(slots<F>(P), fn.f(x.x), ldP_t<kCG>(P + x.x), fn.f(x.y), ldP_t<kCG>(P + x.y));
+  if (log && r.hooked != kNoHook) log_hook(log, r.hooked);
+}
+
 struct WarpRing {
   uint32_t *cu, *pu, *cv, *pv;
   uint32_t *Z;    // zero-tree bitmap, or null

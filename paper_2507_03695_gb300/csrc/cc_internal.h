@@ -40,6 +40,7 @@ struct alignas(128) Ctrl {
   unsigned long long stats[4];  // optional edge-pass counters
   unsigned long long work;      // edge pass, dynamic schedule: steps claimed so far
   unsigned long long pairs;     // cc_forest_pairs: non-root vertices found
+  uint32_t ref;                 // edge pass by bits: root name of the reference tree
 };
 static_assert(offsetof(Ctrl, q_u) % 8 == 0, "the query pair is loaded with an 8-byte access");
 static_assert(offsetof(Ctrl, maxkey) % 8 == 0 && offsetof(Ctrl, ncomp) % 8 == 0, "64-bit atomics");
@@ -275,6 +276,18 @@ cudaError_t launch_edge_pass(bool rf, int filter, int ept, int block, const Edge
 // dyn: warps claim their edges from a counter in ctrl (reset on s before the
 // launch), so at most one dynamic edge pass per Ctrl may be in flight.
 // Sets *reject (ctrl->reject when null) and the range error bit when an id is >= n.
+// The edge pass by vertex bits in shared memory (cc_bits.cu), right after init:
+// graphs of at most kBitsVertices vertices (196,608 bytes of bits) and at
+// least kBitsMinDegree edges per vertex (sparser ones have no giant component
+// to speak of: a grid's 1.8 edges per vertex took 1.3 times as long) and
+// kBitsMinEdges in all (below, its launches are most of the time).
+// bits: bits_bytes(n) bytes, 16-byte aligned.
+constexpr uint64_t kBitsVertices = 1536ULL << 10;
+constexpr uint64_t kBitsMinEdges = 1ULL << 15, kBitsMaxEdges = 1ULL << 36, kBitsMinDegree = 3;
+constexpr size_t bits_bytes(uint64_t n) { return (size_t)((n + 127) / 128 * 16); }
+bool bits_pass_fits(uint64_t n_vertices, uint64_t n_edges);
+cudaError_t launch_edge_pass_bits(bool rf, const EdgeSpan &e, uint32_t *P, uint32_t n, Ctrl *ctrl, uint32_t *bits,
+                                  cudaStream_t s);
 cudaError_t launch_validate(const EdgeSpan &e, uint32_t n, Ctrl *ctrl, cudaStream_t s, uint32_t *reject = nullptr);
 cudaError_t launch_flatten(bool rf, int label_space, uint32_t *P, uint32_t n, uint32_t *L, Ctrl *ctrl,
                            cudaStream_t s);

@@ -68,25 +68,6 @@ __global__ void __launch_bounds__(256) k_init(uint32_t *__restrict__ P, uint32_t
 
 // --------------------------------------------------------------- edge pass
 
-// Range check of one edge; an out-of-range id flags the error and turns the
-// edge into the no-op self-loop (0, 0).
-__device__ __forceinline__ void guard(uint32_t &a, uint32_t &b, uint32_t n, Ctrl *ctrl) {
-  if (a >= n || b >= n) {
-    set_err(ctrl, kErrRange);
-    a = 0u;
-    b = 0u;
-  }
-}
-
-template <class F>
-__device__ __forceinline__ void single_edge(uint32_t *P, const F fn, const uint2 *e, uint32_t n,
-                                            Ctrl *ctrl, uint32_t *log = nullptr) {
-  uint2 x = ld_edge(e);
-  guard(x.x, x.y, n, ctrl);
-  const UniteResult r = unite(slots<F>(P), fn.f(x.x), ldP(P + x.x), fn.f(x.y), ldP(P + x.y));
-  if (log && r.hooked != kNoHook) log_hook(log, r.hooked);
-}
-
 // Direct form: each thread takes Q 128-bit loads (2Q edges) per iteration,
 // issues all 4Q parent loads together, then resolves its edges one by one.
 template <class F, int Q>
