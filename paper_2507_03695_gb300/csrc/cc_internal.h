@@ -146,7 +146,7 @@ inline uint32_t cert_sample_stride(uint64_t n_edges) {
   const uint64_t s = n_edges >> 19;
   return s > kCertSample ? (uint32_t)(s < 4096 ? s : 4096) : kCertSample;
 }
-struct CertScratch {
+struct alignas(16) CertScratch {
   unsigned long long owner[kCertBuckets];   // per bucket, its best sampled (count << 32) | ~vertex; 0 = none
   unsigned long long top[kCertTop];         // the best owners, same packing; 0 = empty slot
   unsigned long long top_cnt[kCertTop];     // their exact degrees
@@ -155,6 +155,7 @@ struct CertScratch {
   unsigned int sel_done;                    // candidate-selection blocks finished (the last one ranks)
   unsigned int list_n[kListSegs];           // per list segment, vertices appended (may exceed its room)
   unsigned int blocks_done;                 // counting blocks finished (the last one decides)
+  unsigned int bucket_shift;                // log2 of the owner buckets that the counting pass takes as one
   // Initial Push (Algorithm 4): neighbours of the sampled argmax m', appended
   // through kPushLanes counters, each owning a segment of the push buffer
   unsigned int push_cnt[256];

@@ -523,11 +523,14 @@ __global__ void __launch_bounds__(256) k_validate(const uint4 *__restrict__ e4, 
 __global__ void __launch_bounds__(256) k_gmin_probe(uint32_t *P, uint32_t n, Ctrl *ctrl) {
   const RootR fn = RootR::load(ctrl);
   const uint32_t m = fn.m;
-  __shared__ uint32_t s_stop;
+  __shared__ uint32_t s_stop, s_best;
   const uint64_t chunk = 4ull * blockDim.x;
   for (uint64_t c = blockIdx.x;; c += gridDim.x) {
     const uint64_t start = c * chunk;
-    if (threadIdx.x == 0) s_stop = (start >= m) || (start > ld_volatile_u32(&ctrl->gmin));
+    if (threadIdx.x == 0) {
+      s_stop = (start >= m) || (start > ld_volatile_u32(&ctrl->gmin));
+      s_best = 0xFFFFFFFFu;
+    }
     __syncthreads();
     const bool stop = s_stop;
     __syncthreads();
@@ -541,9 +544,27 @@ __global__ void __launch_bounds__(256) k_gmin_probe(uint32_t *P, uint32_t n, Ctr
         if (root_name(slots<RootR>(P), fn.f((uint32_t)v), pv) == 0u) best = (uint32_t)v;
       }
     }
+    // one global atomic per block and chunk at most: the first chunks nearly
+    // always hold the answer, and an atomic per warp of the whole grid on the
+    // one word took longer than the scan (R-MAT scale 20: 9.9 us, 24: 14.3)
     best = __reduce_min_sync(0xFFFFFFFFu, best);
-    if ((threadIdx.x & 31) == 0 && best != 0xFFFFFFFFu) atomicMin(&ctrl->gmin, best);
+    if ((threadIdx.x & 31) == 0 && best != 0xFFFFFFFFu) atomicMin(&s_best, best);
+    __syncthreads();
+    if (threadIdx.x == 0 && s_best < ld_volatile_u32(&ctrl->gmin)) atomicMin(&ctrl->gmin, s_best);
   }
+}
+
+// Adds the block's roots to ctrl->ncomp, one global atomic per block: one per
+// warp met on the one word for longer than a small flatten takes (R-MAT scale
+// 20, flatten: 16.3 us). Every thread of the block calls it.
+__device__ __forceinline__ void add_roots(unsigned long long roots, Ctrl *ctrl) {
+  __shared__ unsigned long long s_roots;
+  if (threadIdx.x == 0) s_roots = 0ULL;
+  __syncthreads();
+  roots = warp_sum_u64(roots);
+  if ((threadIdx.x & 31) == 0 && roots) atomicAdd(&s_roots, roots);
+  __syncthreads();
+  if (threadIdx.x == 0 && s_roots) atomicAdd(&ctrl->ncomp, s_roots);
 }
 
 // Pointer jumping (Algorithm 3): every vertex finds its root name c with
@@ -656,8 +677,7 @@ __global__ void __launch_bounds__(256) k_flatten4(uint32_t *P, uint32_t n, uint3
     if (c != pv) stP(P + v, c);
     if (L) L[v] = label_of<F, LABEL>(c, gmin);
   }
-  roots = warp_sum_u64(roots);
-  if ((threadIdx.x & 31) == 0 && roots) atomicAdd(&ctrl->ncomp, roots);
+  add_roots(roots, ctrl);
 }
 
 // One vertex per thread, for label buffers that are not 16-byte aligned.
@@ -677,8 +697,7 @@ __global__ void __launch_bounds__(256) k_flatten(uint32_t *P, uint32_t n, uint32
     if (c != pv) stP(P + v, c);
     if (L) __stcs(L + v, label_of<F, LABEL>(c, gmin));
   }
-  roots = warp_sum_u64(roots);
-  if ((threadIdx.x & 31) == 0 && roots) atomicAdd(&ctrl->ncomp, roots);
+  add_roots(roots, ctrl);
 }
 
 template <class F>
@@ -689,8 +708,7 @@ __global__ void __launch_bounds__(256) k_count_roots(const uint32_t *__restrict_
   for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n;
        i += (uint64_t)gridDim.x * blockDim.x)
     roots += (P[i] == fn.f((uint32_t)i));
-  roots = warp_sum_u64(roots);
-  if ((threadIdx.x & 31) == 0 && roots) atomicAdd(&ctrl->ncomp, roots);
+  add_roots(roots, ctrl);
 }
 
 template <class F>

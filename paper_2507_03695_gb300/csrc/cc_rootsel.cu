@@ -51,6 +51,25 @@ __global__ void __launch_bounds__(256) k_zero_cnt(C *cnt, uint32_t n, const uint
     cnt[v] = (C)0;
 }
 
+// Clears what a certified selection starts from: the n sampled counters, the
+// scratch and the control fields, in one launch (five memsets took 7 us of a
+// small run).
+__global__ void __launch_bounds__(256) k_select_begin(uint32_t *cnt, uint32_t n, CertScratch *cs, Ctrl *ctrl) {
+  const uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x, T = (uint64_t)gridDim.x * blockDim.x;
+  const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+  for (uint64_t i = t; i < n / 4u; i += T) reinterpret_cast<uint4 *>(cnt)[i] = zero;
+  if (t < (n & 3u)) cnt[n - 1u - (uint32_t)t] = 0u;
+  static_assert(sizeof(CertScratch) % 16 == 0 && alignof(CertScratch) >= 16, "cleared 16 bytes at a time");
+  for (uint64_t i = t; i < sizeof(CertScratch) / 16; i += T) reinterpret_cast<uint4 *>(cs)[i] = zero;
+  if (t == 0) {
+    ctrl->maxkey = 0ULL;
+    ctrl->maxcnt = 0ULL;
+    ctrl->m_sel = 0xFFFFFFFFu;
+    ctrl->n_cand = 0u;
+    ctrl->cert = 0u;
+  }
+}
+
 // Edge idx lies in a sampled group of k_degree_sampled (1 group of
 // kSampleGroup in stride, counted from the start of the edge array); stride
 // 0: never.
@@ -205,8 +224,10 @@ __global__ void k_finalize_m(Ctrl *ctrl, const uint32_t *skip) {
 // One multiplicative hash picks the bucket (13 bits) of a vertex. Each bucket
 // has at most one candidate, its owner; every other vertex of the bucket is
 // counted in the bucket's total.
-__device__ __forceinline__ uint32_t bucket_of(uint32_t x) { return (x * 2654435769u) >> 19; }
-static_assert(kCertBuckets == 8192, "13-bit buckets");
+constexpr uint32_t kBucketShift = 19;
+static_assert(kCertBuckets == 1u << (32 - kBucketShift), "13-bit buckets");
+__device__ __forceinline__ uint32_t bucket_hash(uint32_t x) { return x * 2654435769u; }
+__device__ __forceinline__ uint32_t bucket_of(uint32_t x) { return bucket_hash(x) >> kBucketShift; }
 
 // Candidates: every vertex whose sampled count is at least 1/32 of the largest
 // competes for its bucket; the larger sampled count (then the smaller id)
@@ -217,11 +238,13 @@ static_assert(kCertBuckets == 8192, "13-bit buckets");
 // ranks the owners and keeps the kCertTop best for the counting pass.
 // kList: the vertices are those appended to the list's segments (as many as
 // each segment holds), else every vertex 0 .. n-1.
+constexpr int kSelectBlock = 1024, kSelectBlocks = (int)kListSegs;  // the list form's launch
+
 template <bool kList>
-__global__ void __launch_bounds__(256) k_select_candidates(const uint32_t *__restrict__ cnt, uint32_t n,
+__global__ void __launch_bounds__(kList ? kSelectBlock : 256) k_select_candidates(const uint32_t *__restrict__ cnt, uint32_t n,
                                                            Ctrl *ctrl, CertScratch *cs,
                                                            const uint32_t *__restrict__ list, uint32_t list_cap,
-                                                           WideHot *wide_hot, uint32_t s_bits, uint32_t ways) {
+                                                           WideHot *wide_hot, uint32_t s_bits, uint32_t ways, uint64_t sampled) {
   const uint32_t cmax = (uint32_t)(*(volatile unsigned long long *)&ctrl->maxkey >> 32);
   if (cmax < 64u) return;  // uniform over the grid: no block ranks, top stays empty
   const uint32_t thr = cmax >> 5;
@@ -289,6 +312,15 @@ __global__ void __launch_bounds__(256) k_select_candidates(const uint32_t *__res
       loc[k] = hi;
     }
   }
+  // The counting pass may take several owner buckets as one: the proof needs
+  // the buckets' totals well below the best candidate's degree, here 1/16 on
+  // average, and every block clears and adds up its buckets (R-MAT scale 16
+  // takes 2048 of them, scale 20 4096, scale 24 all 8192).
+  if (threadIdx.x == 0) {
+    uint32_t shift = 0;
+    while (sampled && shift < 3u && (kCertBuckets >> (shift + 1u)) * (uint64_t)cmax >= 16u * sampled) ++shift;
+    cs->bucket_shift = shift;
+  }
   uint32_t next = 0;  // loc[next] is this thread's best untaken key
   for (uint32_t r = 0; r < kCertTop; ++r) {
     unsigned long long mine = 0ULL;
@@ -345,11 +377,12 @@ __device__ void certify_decide_block(const CertScratch *cs, Ctrl *ctrl) {
     const unsigned long long key = (cc[k] << 32) | (uint32_t)o;  // low half: ~vertex
     best = key > best ? key : best;
   }
-  for (uint32_t b = threadIdx.x; b < kCertBuckets && !skip && any; b += blockDim.x) {
+  const uint32_t shift = __ldcg(&cs->bucket_shift);
+  for (uint32_t b = threadIdx.x; b < (kCertBuckets >> shift) && !skip && any; b += blockDim.x) {
     unsigned long long t = __ldcg(&cs->bucket[b]);
 #pragma unroll
     for (uint32_t k = 0; k < kCertTop; ++k)
-      if (cc[k] && bucket_of(cv[k]) == b) t -= cc[k];
+      if (cc[k] && (bucket_of(cv[k]) >> shift) == b) t -= cc[k];
     bound = t > bound ? t : bound;
   }
   bound = block_max_u64(bound);
@@ -401,14 +434,19 @@ struct CertCounter {
   uint32_t key[kCertTop];  // candidate ids (an empty slot matches only id 2^32 - 1, and is ignored)
   uint32_t c[kCertTop];
   uint32_t *bk;
+  uint32_t shift;  // of the hash: kBucketShift + CertScratch::bucket_shift
   __device__ __forceinline__ void operator()(uint32_t x) {
-    atomicAdd(&bk[bucket_of(x)], 1u);
+    atomicAdd(&bk[bucket_hash(x) >> shift], 1u);
 #pragma unroll
     for (uint32_t k = 0; k < kCertTop; ++k) c[k] += x == key[k] ? 1u : 0u;
   }
 };
 
+// Every block clears and adds up all buckets, so a thread gets at least 16
+// edge loads. (Blocks of 1024 threads, half as many, would not fit beside the
+// serving executor's blocks.)
 constexpr int kCertBlock = 512;
+constexpr uint64_t kCertQuadsPerBlock = 16ull * kCertBlock;
 
 __global__ void __launch_bounds__(kCertBlock, 2)
     k_degree_certify(const uint4 *__restrict__ e4, uint64_t n_quads, const uint2 *head, const uint2 *tail, uint32_t n,
@@ -423,6 +461,8 @@ __global__ void __launch_bounds__(kCertBlock, 2)
   }
   CertCounter cnt;
   cnt.bk = csm;
+  const uint32_t merged = *(const volatile unsigned int *)&cs->bucket_shift, buckets = kCertBuckets >> merged;
+  cnt.shift = kBucketShift + merged;
 #pragma unroll
   for (uint32_t k = 0; k < kCertTop; ++k) {
     const unsigned long long o = *(const volatile unsigned long long *)&cs->top[k];
@@ -432,7 +472,7 @@ __global__ void __launch_bounds__(kCertBlock, 2)
   // the sampled argmax, whose neighbours the push list gathers
   const uint32_t mp = ~(uint32_t)(*(const volatile unsigned long long *)&ctrl->maxkey);
   if (push_buf && blockIdx.x == 0 && threadIdx.x == 0) cs->push_m = mp + 1u;
-  for (uint32_t i = threadIdx.x; i < kCertBuckets; i += blockDim.x) csm[i] = 0u;
+  for (uint32_t i = threadIdx.x; i < buckets; i += blockDim.x) csm[i] = 0u;
   __syncthreads();
   const uint64_t pol = policy_evict_first();
   const uint64_t T = (uint64_t)gridDim.x * blockDim.x;
@@ -483,7 +523,7 @@ __global__ void __launch_bounds__(kCertBlock, 2)
     if ((threadIdx.x & 31) == 0 && w) atomicAdd(&cs->top_cnt[k], (unsigned long long)w);
   }
   __syncthreads();
-  for (uint32_t i = threadIdx.x; i < kCertBuckets; i += blockDim.x)
+  for (uint32_t i = threadIdx.x; i < buckets; i += blockDim.x)
     if (csm[i]) atomicAdd(&cs->bucket[i], (unsigned long long)csm[i]);
   if (!decide) return;
   __shared__ unsigned s_last;
@@ -590,11 +630,10 @@ cudaError_t launch_root_select_certified(const uint32_t *edges, uint64_t n_edges
   const uint32_t s_bits = id_bits(n);
   if (!list || list_cap < kListSegs || list_cap % kListSegs) list = nullptr;
   // 0. reset the sampled counters, the scratch and the control fields
-  if ((err = cudaMemsetAsync(cnt, 0, (size_t)n * sizeof(uint32_t), s)) != cudaSuccess) return err;
-  if ((err = cudaMemsetAsync(cs, 0, sizeof(CertScratch), s)) != cudaSuccess) return err;
-  if ((err = cudaMemsetAsync(&ctrl->maxkey, 0, 2 * sizeof(unsigned long long), s)) != cudaSuccess) return err;
-  if ((err = cudaMemsetAsync(&ctrl->m_sel, 0xFF, sizeof(uint32_t), s)) != cudaSuccess) return err;
-  if ((err = cudaMemsetAsync(&ctrl->n_cand, 0, 2 * sizeof(uint32_t), s)) != cudaSuccess) return err;
+  const uint64_t words = (uint64_t)n / 4u + sizeof(CertScratch) / 16u;
+  const unsigned gz0 = clamp_grid((words + 255) / 256, persistent_cap((const void *)k_select_begin, 256, 0));
+  k_select_begin<<<gz0, 256, 0, s>>>(static_cast<uint32_t *>(cnt), n, cs, ctrl);
+  note_launch();
   if (!list) wide_hot = nullptr;
   if (wide_hot && (err = cudaMemsetAsync(wide_hot->slot, 0, wide_ways(s_bits) * sizeof(wide_hot->slot[0]), s)) != cudaSuccess) return err;
   uint32_t *c32 = static_cast<uint32_t *>(cnt);
@@ -608,12 +647,12 @@ cudaError_t launch_root_select_certified(const uint32_t *edges, uint64_t n_edges
   if (push_buf && (err = launch_argmax_u32(c32, n, ctrl, s)) != cudaSuccess) return err;
   // 2. candidates: the owners of their buckets, from the list when there is one
   if (list) {
-    k_select_candidates<true><<<kListSegs, 256, 0, s>>>(c32, n, ctrl, cs, list, list_cap, wide_hot,
-                                                s_bits, wide_hot ? wide_ways(s_bits) : 0u);
+    k_select_candidates<true><<<kSelectBlocks, kSelectBlock, 0, s>>>(c32, n, ctrl, cs, list, list_cap, wide_hot,
+                                                s_bits, wide_hot ? wide_ways(s_bits) : 0u, 2 * (n_edges / stride + 1));
   } else {
     const unsigned gsel = clamp_grid(((uint64_t)n + 255) / 256,
                                      persistent_cap((const void *)k_select_candidates<false>, 256, 0));
-    k_select_candidates<false><<<gsel, 256, 0, s>>>(c32, n, ctrl, cs, nullptr, 0u, nullptr, 0u, 0u);
+    k_select_candidates<false><<<gsel, 256, 0, s>>>(c32, n, ctrl, cs, nullptr, 0u, nullptr, 0u, 0u, 0u);
   }
   note_launch();
   if (wide_hot) {
@@ -625,7 +664,7 @@ cudaError_t launch_root_select_certified(const uint32_t *edges, uint64_t n_edges
   if ((err = ensure_func_attr((const void *)k_degree_certify, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)kCertSmem, smem_set_certify)) != cudaSuccess)
     return err;
-  const unsigned gcert = clamp_grid((e.n_quads + kCertBlock - 1) / kCertBlock,
+  const unsigned gcert = clamp_grid((e.n_quads + kCertQuadsPerBlock - 1) / kCertQuadsPerBlock,
                                     persistent_cap((const void *)k_degree_certify, kCertBlock, kCertSmem));
   // 4. the proof: taken by the counting pass's last block (which also
   // gathers the push list when asked to)
@@ -724,7 +763,7 @@ cudaError_t chunked_select_begin(const uint32_t *chunk0, uint64_t n0, void *cnt,
   if ((err = launch_argmax_u32(c32, n, ctrl, s)) != cudaSuccess) return err;
   const unsigned gsel = clamp_grid(((uint64_t)n + 255) / 256,
                                    persistent_cap((const void *)k_select_candidates<false>, 256, 0));
-  k_select_candidates<false><<<gsel, 256, 0, s>>>(c32, n, ctrl, cs, nullptr, 0u, nullptr, 0u, 0u);
+  k_select_candidates<false><<<gsel, 256, 0, s>>>(c32, n, ctrl, cs, nullptr, 0u, nullptr, 0u, 0u, 0u);
   note_launch();
   k_spec_begin<<<1, 1, 0, s>>>(ctrl);
   note_launch();
@@ -745,7 +784,7 @@ cudaError_t chunked_select_chunk(const EdgeSpan &chunk, bool first, void *cnt, b
                               (int)kCertSmem, smem_set_certify)) != cudaSuccess)
     return err;
   const unsigned gcert =
-      clamp_grid((chunk.n_quads + kCertBlock - 1) / kCertBlock,
+      clamp_grid((chunk.n_quads + kCertQuadsPerBlock - 1) / kCertQuadsPerBlock,
                  persistent_cap((const void *)k_degree_certify, kCertBlock, kCertSmem));
   k_degree_certify<<<gcert, kCertBlock, kCertSmem, s>>>(chunk.quads, chunk.n_quads, chunk.head, chunk.tail, n, cs,
                                                         ctrl, 0, nullptr, 0u);
