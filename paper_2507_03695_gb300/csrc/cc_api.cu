@@ -38,6 +38,7 @@ struct cc_graph {
   size_t ev_cur = 0;                                 // set of the current run
   bool timed_run = false;
   bool ncomp_fresh = false;
+  uint64_t applied = 0;  // edges of the last run and of the inserts after it
   uint64_t owned = 0;
   uint32_t *csr_rows = nullptr;  // cc_run_csr: the row of each tile's first entry
   uint64_t csr_rows_cap = 0;
@@ -427,6 +428,7 @@ cc_status cc_run(cc_graph *g, const uint32_t *edges_dev, uint64_t n_edges, uint3
   cudaStream_t s = (cudaStream_t)stream;
   g->last = s;
   if (g->n == 0) return CC_OK;
+  g->applied = n_edges;
   const uint32_t n = (uint32_t)g->n;
   const cc::EdgeSpan span = cc::split_edges(edges_dev, n_edges);
   begin_timed_run(g);
@@ -480,6 +482,7 @@ static cc_status run_host_impl(cc_graph *g, const void *edges_host, uint64_t n_e
   g->last = s;
   if (g->n == 0) return CC_OK;
   const uint32_t n = (uint32_t)g->n;
+  g->applied = n_edges;
   if (L_out_host && !g->label_dev) CC_TRY(dev_alloc(g, (void **)&g->label_dev, (size_t)n * 4));
   // When m is known before the edges arrive (identity, or a hint), the edge
   // pass runs on each chunk as soon as it lands. Exact selection takes the
@@ -582,6 +585,7 @@ cc_status cc_run_csr(cc_graph *g, const uint64_t *offsets_dev, const uint32_t *n
   g->last = s;
   if (g->n == 0) return CC_OK;
   const uint32_t n = (uint32_t)g->n;
+  g->applied = n_entries;
   const uint64_t tiles = cc::csr_tiles(n_entries);
   if (tiles > g->csr_rows_cap) {
     CC_TRY(cudaStreamSynchronize(s));
@@ -661,16 +665,24 @@ cc_status cc_stream_insert(cc_graph *g, const uint32_t *edges_dev, uint64_t n_ed
   g->last = s;
   if (g->n == 0 || n_edges == 0) return CC_OK;
   const cc::EdgeSpan span = cc::split_edges(edges_dev, n_edges);
+  // Trees are taken to be settled once the handle has seen two edges per
+  // vertex: most inserted pairs then end at the filter or after one hook.
+  const bool settled = g->applied >= 2 * g->n;
+  g->applied += n_edges;
+  g->ncomp_fresh = false;
+  if (n_edges <= cc::kInsertOneBlock)
+    return from_cuda(cc::launch_insert_small(g->rf, span, g->P, (uint32_t)g->n, g->ctrl, s));
   CC_TRY(cudaMemsetAsync(&g->ctrl->reject, 0, sizeof(uint32_t), s));
   CC_TRY(cc::launch_validate(span, (uint32_t)g->n, g->ctrl, s));
   uint32_t *Z = (g->z && (g->z_forced || g->z_auto_ok)) ? g->z : nullptr;
   const uint32_t *zsel = (Z && !g->z_forced) ? &g->ctrl->cert : nullptr;
-  // the last run's certificate (when its exact selection ran) picks the form
-  const uint32_t *hub = g->z_auto_ok ? &g->ctrl->cert : nullptr;
-  CC_TRY(cc::launch_edge_pass(g->rf, eff_filter(g), eff_ept(g), eff_block(g), span, g->P,
-                              (uint32_t)g->n, g->ctrl, &g->ctrl->reject, s, Z, zsel, false, nullptr, hub, true,
-                              g->z_auto_ok ? g->cert->hot : nullptr));
-  g->ncomp_fresh = false;
+  // the last run's certificate (when its exact selection ran) picks the form;
+  // a short list into settled trees takes the form for any graph, one launch
+  const bool brief = settled && !Z && n_edges < (1ULL << 20);
+  const uint32_t *hub = g->z_auto_ok && !brief ? &g->ctrl->cert : nullptr;
+  CC_TRY(cc::launch_edge_pass(g->rf, eff_filter(g), eff_ept(g), eff_block(g), span, g->P, (uint32_t)g->n, g->ctrl,
+                              &g->ctrl->reject, s, Z, zsel, false, nullptr, hub, !brief,
+                              g->z_auto_ok ? g->cert->hot : nullptr, nullptr, settled));
   return CC_OK;
 }
 
@@ -843,6 +855,7 @@ cc_status cc_restore(cc_graph *g, const void *host_buf, uint64_t bytes) {
   if (g->n) CC_TRY(cudaMemcpy(g->P, (const char *)host_buf + sizeof(h), g->n * 4, cudaMemcpyHostToDevice));
   g->host_ctrl->m = h.m;
   CC_TRY(cudaMemcpy(&g->ctrl->m, &g->host_ctrl->m, sizeof(uint32_t), cudaMemcpyHostToDevice));
+  g->applied = 0;
   if (g->z) CC_TRY(cudaMemset(g->z, 0, g->z_bytes));  // the restored P has its own trees
   g->z_auto_ok = false;
   g->ncomp_fresh = false;

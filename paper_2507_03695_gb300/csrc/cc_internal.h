@@ -273,7 +273,14 @@ cudaError_t launch_edge_pass(bool rf, int filter, int ept, int block, const Edge
                              uint32_t n, Ctrl *ctrl, const uint32_t *skip, cudaStream_t s,
                              uint32_t *Z = nullptr, const uint32_t *zsel = nullptr, bool one_shot = false,
                              uint32_t *log = nullptr, const uint32_t *hub = nullptr, bool dyn = false,
-                             const unsigned long long *hot = nullptr, const WideHot *wide_hot = nullptr);
+                             const unsigned long long *hot = nullptr, const WideHot *wide_hot = nullptr,
+                             bool settled = false);
+// settled: the trees exist already, so the grid need not be kept small for the
+// edges that would all meet on the first roots.
+// An insert of at most kInsertOneBlock pairs: validation and hooking in one
+// block.
+constexpr uint64_t kInsertOneBlock = 4096;
+cudaError_t launch_insert_small(bool rf, const EdgeSpan &e, uint32_t *P, uint32_t n, Ctrl *ctrl, cudaStream_t s);
 // dyn: warps claim their edges from a counter in ctrl (reset on s before the
 // launch), so at most one dynamic edge pass per Ctrl may be in flight.
 // Sets *reject (ctrl->reject when null) and the range error bit when an id is >= n.

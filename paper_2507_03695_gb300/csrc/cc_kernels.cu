@@ -515,6 +515,39 @@ __global__ void __launch_bounds__(256) k_validate(const uint4 *__restrict__ e4, 
   }
 }
 
+// A short insert in one block: every thread holds its pairs (at most 4) while
+// the block validates them, then hooks them. Four launches and two memsets
+// otherwise took longer than the work.
+constexpr int kInsertBlock = 1024;
+static_assert(kInsertOneBlock <= 4 * kInsertBlock, "four pairs per thread");
+
+template <class F>
+__global__ void __launch_bounds__(kInsertBlock) k_insert_small(const uint2 *__restrict__ e, uint32_t n_edges,
+                                                               uint32_t *P, uint32_t n, Ctrl *ctrl) {
+  const F fn = F::load(ctrl);
+  uint32_t *const S = slots<F>(P);
+  uint2 x[4];
+  bool bad = false;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const uint32_t i = threadIdx.x + (uint32_t)j * kInsertBlock;
+    x[j] = i < n_edges ? ld_edge(e + i) : make_uint2(0u, 0u);
+    bad |= x[j].x >= n || x[j].y >= n;
+  }
+  if (__syncthreads_or(bad)) {  // nothing is applied
+    if (threadIdx.x == 0) set_err(ctrl, kErrRange);
+    return;
+  }
+  uint32_t p[8];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    p[2 * j] = ldP_cg(P + x[j].x);
+    p[2 * j + 1] = ldP_cg(P + x[j].y);
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) unite<true>(S, fn.f(x[j].x), p[2 * j], fn.f(x[j].y), p[2 * j + 1]);
+}
+
 // ------------------------------------------------------------------ flatten
 
 // Smallest vertex whose root value is 0 under R. Its answer is at most m, so
@@ -901,7 +934,7 @@ template <class F, int Q>
 cudaError_t edge_pass_q(int filter, int block, const EdgeSpan &e, uint32_t *P, uint32_t n, Ctrl *ctrl,
                         const uint32_t *skip, uint32_t *Z, const uint32_t *zsel, bool one_shot, uint32_t *log,
                         const uint32_t *hub, bool dyn, cudaStream_t s, const unsigned long long *hot,
-                        const WideHot *wide_hot) {
+                        const WideHot *wide_hot, bool settled) {
   const uint64_t per_block = (uint64_t)block * Q;
   // At least kMinWaves grid iterations per thread: when a whole graph fits
   // one wave, every edge reads P before any hooking and duplicate hub edges
@@ -909,7 +942,10 @@ cudaError_t edge_pass_q(int filter, int block, const EdgeSpan &e, uint32_t *P, u
   // later waves find most edges already joined. one_shot: no cap at the
   // resident blocks, so blocks retire after their kMinWaves iterations and
   // kernels of other streams get SMs while this one runs.
-  const uint64_t want = (e.n_quads + per_block * kMinWaves - 1) / (per_block * kMinWaves);
+  // Into settled trees one iteration per thread does: ten inserts of 10^3 to
+  // 10^6 pairs into R-MAT scale 20 took 51 us each on 1 to 62 blocks.
+  const uint64_t per = per_block * (settled ? 1 : kMinWaves);
+  const uint64_t want = (e.n_quads + per - 1) / per;
   const uint64_t cap_big = 0x7FFFFFFFull;
   if (filter) {
     unsigned long long *work = nullptr;
@@ -985,11 +1021,11 @@ template <class F>
 cudaError_t edge_pass_f(int filter, int ept, int block, const EdgeSpan &e, uint32_t *P, uint32_t n,
                         Ctrl *ctrl, const uint32_t *skip, uint32_t *Z, const uint32_t *zsel, bool one_shot,
                         uint32_t *log, const uint32_t *hub, bool dyn, cudaStream_t s, const unsigned long long *hot,
-                        const WideHot *wide_hot) {
+                        const WideHot *wide_hot, bool settled) {
   switch (ept) {
-    case 2: return edge_pass_q<F, 1>(filter, block, e, P, n, ctrl, skip, Z, zsel, one_shot, log, hub, dyn, s, hot, nullptr);
-    case 8: return edge_pass_q<F, 4>(filter, block, e, P, n, ctrl, skip, Z, zsel, one_shot, log, hub, dyn, s, hot, nullptr);
-    default: return edge_pass_q<F, 2>(filter, block, e, P, n, ctrl, skip, Z, zsel, one_shot, log, hub, dyn, s, hot, wide_hot);
+    case 2: return edge_pass_q<F, 1>(filter, block, e, P, n, ctrl, skip, Z, zsel, one_shot, log, hub, dyn, s, hot, nullptr, settled);
+    case 8: return edge_pass_q<F, 4>(filter, block, e, P, n, ctrl, skip, Z, zsel, one_shot, log, hub, dyn, s, hot, nullptr, settled);
+    default: return edge_pass_q<F, 2>(filter, block, e, P, n, ctrl, skip, Z, zsel, one_shot, log, hub, dyn, s, hot, wide_hot, settled);
   }
 }
 }  // namespace
@@ -997,20 +1033,31 @@ cudaError_t edge_pass_f(int filter, int ept, int block, const EdgeSpan &e, uint3
 cudaError_t launch_edge_pass(bool rf, int filter, int ept, int block, const EdgeSpan &e, uint32_t *P,
                              uint32_t n, Ctrl *ctrl, const uint32_t *skip, cudaStream_t s, uint32_t *Z,
                              const uint32_t *zsel, bool one_shot, uint32_t *log, const uint32_t *hub, bool dyn,
-                             const unsigned long long *hot, const WideHot *wide_hot) {
+                             const unsigned long long *hot, const WideHot *wide_hot, bool settled) {
   if (block != 128 && block != 256 && block != 512) block = 256;
   if (e.n_quads == 0 && !e.head && !e.tail) return cudaSuccess;
   if (log) filter = 1;  // the log is kept by the filtered form
   return rf ? edge_pass_f<RootR>(filter, ept, block, e, P, n, ctrl, skip, Z, zsel, one_shot, log, hub, dyn, s, hot,
-                                   wide_hot)
+                                   wide_hot, settled)
             : edge_pass_f<RootId>(filter, ept, block, e, P, n, ctrl, skip, Z, zsel, one_shot, log, hub, dyn, s,
-                                  nullptr, nullptr);
+                                  nullptr, nullptr, settled);
 }
 
 cudaError_t launch_validate(const EdgeSpan &e, uint32_t n, Ctrl *ctrl, cudaStream_t s, uint32_t *reject) {
   if (e.n_quads == 0 && !e.head && !e.tail) return cudaSuccess;
   const unsigned g = clamp_grid((e.n_quads + 255) / 256, persistent_cap((const void *)k_validate, 256, 0));
   k_validate<<<g, 256, 0, s>>>(e.quads, e.n_quads, e.head, e.tail, n, ctrl, reject ? reject : &ctrl->reject);
+  note_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t launch_insert_small(bool rf, const EdgeSpan &e, uint32_t *P, uint32_t n, Ctrl *ctrl, cudaStream_t s) {
+  const uint2 *first = e.head ? e.head : (e.n_quads ? reinterpret_cast<const uint2 *>(e.quads) : e.tail);
+  const uint32_t count = (uint32_t)(2 * e.n_quads + (e.head ? 1 : 0) + (e.tail ? 1 : 0));
+  if (rf)
+    k_insert_small<RootR><<<1, kInsertBlock, 0, s>>>(first, count, P, n, ctrl);
+  else
+    k_insert_small<RootId><<<1, kInsertBlock, 0, s>>>(first, count, P, n, ctrl);
   note_launch();
   return cudaGetLastError();
 }
