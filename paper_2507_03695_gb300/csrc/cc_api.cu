@@ -220,11 +220,17 @@ cudaError_t ensure_cnt(cc_graph *g, bool wide, cudaStream_t s) {
   return cudaSuccess;
 }
 
+// 1: m from the degrees of all edges; k > 1: of one sampled group in k.
+uint32_t select_stride(const cc_graph *g) {
+  const uint32_t stride = g->opt.sample_stride ? (uint32_t)g->opt.sample_stride : 16u;
+  return g->opt.root_select == CC_ROOT_SELECT_SAMPLED && stride > 1 ? stride : 1u;
+}
+
 cc_status root_select(cc_graph *g, const uint32_t *edges, uint64_t n_edges, const cc::EdgeSpan &span,
                       cudaStream_t s, int *m_src) {
   const uint32_t n = (uint32_t)g->n;
-  const uint32_t stride = g->opt.sample_stride ? (uint32_t)g->opt.sample_stride : 16u;
-  const bool sampled = g->opt.root_select == CC_ROOT_SELECT_SAMPLED && stride > 1;
+  const uint32_t stride = select_stride(g);
+  const bool sampled = stride > 1;
   const bool wide = !sampled && n_edges >= (1ULL << 31);
   const size_t need = (size_t)n * (wide ? 8 : 4);
   CC_TRY(ensure_cnt(g, wide, s));
@@ -431,6 +437,16 @@ cc_status cc_run(cc_graph *g, const uint32_t *edges_dev, uint64_t n_edges, uint3
   g->applied = n_edges;
   const uint32_t n = (uint32_t)g->n;
   const cc::EdgeSpan span = cc::split_edges(edges_dev, n_edges);
+  if (g->bits && !g->opt.timing && cc::tiny_fits(n, n_edges)) {  // (timed runs keep their phases apart)
+    const bool select = g->rf && g->opt.root_hint == CC_ROOT_AUTO;
+    const uint32_t hint = g->rf && !select ? (uint32_t)g->opt.root_hint : 0u;
+    CC_TRY(cc::launch_tiny(g->rf, span, g->P, n, g->ctrl, select ? select_stride(g) : 0u, hint, g->opt.label_space,
+                           L_out_dev, s));
+    g->timed_run = false;
+    g->z_auto_ok = select && g->opt.root_select != CC_ROOT_SELECT_SAMPLED;
+    g->ncomp_fresh = true;
+    return CC_OK;
+  }
   begin_timed_run(g);
   record(g, 0, s);
   int m_src = cc::kMFromHint;

@@ -284,6 +284,14 @@ cudaError_t launch_insert_small(bool rf, const EdgeSpan &e, uint32_t *P, uint32_
 // dyn: warps claim their edges from a counter in ctrl (reset on s before the
 // launch), so at most one dynamic edge pass per Ctrl may be in flight.
 // Sets *reject (ctrl->reject when null) and the range error bit when an id is >= n.
+// A whole run in one block (cc_tiny.cu): at most kTinyVertices vertices (192 KB
+// of shared memory) and kTinyEdges edges. count_stride: how m is chosen (0: it
+// is m_hint; 1: degrees of all edges; k: of one sampled group in k). P, the
+// labels (when L is given), ctrl->m, gmin, ncomp and cert are written.
+constexpr uint64_t kTinyVertices = 48ULL << 10, kTinyEdges = (1ULL << 15) - 1;
+bool tiny_fits(uint64_t n_vertices, uint64_t n_edges);
+cudaError_t launch_tiny(bool rf, const EdgeSpan &e, uint32_t *P, uint32_t n, Ctrl *ctrl, uint32_t count_stride,
+                        uint32_t m_hint, int label_space, uint32_t *L, cudaStream_t s);
 // The edge pass by vertex bits in shared memory (cc_bits.cu), right after init:
 // graphs of at most kBitsVertices vertices (196,608 bytes of bits) and at
 // least kBitsMinDegree edges per vertex (sparser ones have no giant component
