@@ -89,6 +89,10 @@ bool wants_wide_hot(const cc_options &o, uint64_t n) {
          cc::wide_hot_fits(n);
 }
 
+cc::WideHot *wide_hot_for(const cc_graph *g, uint64_t n_edges) {
+  return cc::wide_hot_pays(g->n, n_edges, g->z != nullptr) ? g->wide_hot : nullptr;
+}
+
 // The vertex bits of small graphs: the edge pass's default shape.
 bool wants_bits(const cc_options &o, uint64_t n) {
   return n >= 1 && n <= cc::kBitsVertices && o.filter != CC_FILTER_OFF && o.filter != CC_FILTER_BITMAP &&
@@ -244,7 +248,7 @@ cc_status root_select(cc_graph *g, const uint32_t *edges, uint64_t n_edges, cons
     return CC_OK;
   }
   CC_TRY(cc::launch_root_select_certified(edges, n_edges, span, g->cnt, wide, n, g->cert, g->ctrl, s, g->push,
-                                         g->push_cap, g->cand_list, g->cand_cap, g->wide_hot));
+                                         g->push_cap, g->cand_list, g->cand_cap, wide_hot_for(g, n_edges)));
   return CC_OK;
 }
 
@@ -475,7 +479,7 @@ cc_status cc_run(cc_graph *g, const uint32_t *edges_dev, uint64_t n_edges, uint3
   } else {
     CC_TRY(cc::launch_edge_pass(g->rf, eff_filter(g), eff_ept(g), eff_block(g), span, g->P, n, g->ctrl,
                                 nullptr, s, Z, zsel, false, nullptr, exact ? &g->ctrl->cert : nullptr, true,
-                                exact ? g->cert->hot : nullptr, exact ? g->wide_hot : nullptr));
+                                exact ? g->cert->hot : nullptr, exact ? wide_hot_for(g, n_edges) : nullptr));
   }
   record(g, 3, s);
   CC_TRY(cc::launch_flatten(g->rf, g->opt.label_space, g->P, n, L_out_dev, g->ctrl, s));

@@ -289,6 +289,61 @@ __device__ __forceinline__ uint32_t wide_bucket(uint32_t y, uint32_t s_bits) {
   return (y << (32u - s_bits)) >> (32u - kWideBits);
 }
 
+// A block's copy of the wide table in shared memory, 16-byte aligned
+// (kWideBuckets words). A field's flag: this block knows the vertex to be in
+// the tree of name 0.
+struct WideTable {
+  uint32_t *H;
+  uint32_t s_bits, ways, fbits, flag, rmask, ones, highs, down, mul;
+
+  // Every thread of the block calls it; __syncthreads() before the first use.
+  __device__ __forceinline__ void load(uint32_t *smem, const uint32_t *__restrict__ words, uint32_t s, uint32_t w) {
+    H = smem;
+    for (uint32_t i = threadIdx.x; i < kWideBuckets / 4; i += blockDim.x)
+      reinterpret_cast<uint4 *>(H)[i] = __ldg(reinterpret_cast<const uint4 *>(words) + i);
+    s_bits = s;
+    ways = w;
+    fbits = s - kWideBits + 1u;  // identifying bits and flag
+    flag = 1u << (fbits - 1u);
+    rmask = flag - 1u;
+    ones = 0;
+    for (uint32_t k = 0; k < ways; ++k) ones |= 1u << (k * fbits);
+    highs = ones * flag;
+    down = 32u - s;
+    mul = kWideMul << down;  // the product's s bits at the top of the word
+  }
+  // The flag bits of the fields of `word` that hold y's vertex.
+  __device__ __forceinline__ uint32_t holds(uint32_t word, uint32_t y) const {
+    return ~(((word ^ (((y >> down) & rmask) * ones)) | highs) - ones) & highs;
+  }
+  __device__ __forceinline__ bool known(uint32_t x) const {
+    const uint32_t y = x * mul, word = H[y >> (32u - kWideBits)];
+    return (holds(word, y) & word) != 0u;
+  }
+  // x is in the tree of name 0: flags its field, if it has one.
+  __device__ __forceinline__ void learn(uint32_t x) {
+    const uint32_t y = x * mul, word = H[y >> (32u - kWideBits)], found = holds(word, y) & ~word;
+    if (found) atomicOr(H + (y >> (32u - kWideBits)), found);
+  }
+  // Asks `in` about every vertex of this warp's share (of kWarps) that is not flagged yet.
+  template <int kWarps, class In>
+  __device__ __forceinline__ void learn_share(uint32_t n, In in) {
+    constexpr uint32_t kShare = kWideBuckets / kWarps;
+    const uint32_t b0 = (threadIdx.x >> 5) * kShare;
+    for (uint32_t b = b0 + (threadIdx.x & 31u); b < b0 + kShare; b += 32u) {
+      const uint32_t word = H[b];
+      uint32_t found = 0u;
+      for (uint32_t w = 0; w < ways; ++w) {
+        const uint32_t f = word >> (w * fbits);
+        const uint32_t v = (((b << (s_bits - kWideBits)) | (f & rmask)) * kWideInv) & (0xFFFFFFFFu >> down);
+        if ((f & flag) || v >= n) continue;
+        if (in(v)) found |= flag << (w * fbits);
+      }
+      if (found) atomicOr(H + b, found);
+    }
+  }
+};
+
 // A changed-root log: log[0] counts the entries that follow it, the names of
 // the roots hooked since the log was last cleared. Its capacity (one entry
 // per vertex) cannot be exceeded: a root is hooked once.

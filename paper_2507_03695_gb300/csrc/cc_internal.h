@@ -188,6 +188,21 @@ inline uint32_t id_bits(uint64_t n) {
   return s;
 }
 inline bool wide_hot_fits(uint64_t n) { return n >= (1ULL << 22) && n <= (1ULL << 30); }
+// Whether a run of n_edges edges uses it; bitmap: P is beyond the zero-tree
+// threshold. Copying the table and learning cost every block about 50 us, and
+// a table lookup saves a request only if its load would not share one: the
+// first endpoints of a list sorted by source do. Whole runs without -> with
+// it, us, R-MAT, random order / sorted by source:
+//   2^22 vertices  2^26 edges 544 -> 590 sorted, 2^27 1139 -> 867 / 793 -> 766
+//   2^24           2^26 775 -> 731 / 604 -> 647, 2^27 1248 -> 1121 / 906 -> 927,
+//                  2^28 2171 -> 1841 / 1484 -> 1440
+//   2^25 - 1       2^29 4011 -> 4060 sorted (the one size found that pays for it)
+//   bitmap, 2^25   2^27 1645 -> 1600 / 1349 -> 1204
+//           2^26   2^24 736 -> 778, 2^26 1321 -> 1328, 2^27 1945 -> 1927 / 1629 -> 1483
+//           2^28   2^30 12107 -> 11557
+inline bool wide_hot_pays(uint64_t n, uint64_t n_edges, bool bitmap) {
+  return n_edges >= (1ULL << 27) && (bitmap || n_edges / 12 >= n);
+}
 inline uint32_t wide_ways(uint32_t s) {
   const uint32_t w = 32u / (s - kWideBits + 1u);
   return w < kWideMaxWays ? w : kWideMaxWays;

@@ -301,7 +301,8 @@ __global__ void __launch_bounds__(512, Q >= 4 ? (kZ ? 1 : 2) : (kZ ? 2 : (kDirec
 // 128 KB of its shared memory to the table, which answers 32 warps' lookups
 // of the hottest vertices: on R-MAT scale 24 (98K entries) L2 requests fell
 // from 489M to 348M. Edge pass before and after: R-MAT scale 28 31.24 -> 27.5
-// ms, 26 (edge factor 16) 7.64 -> 6.68, 24 1.70 -> 1.47, 22 0.51 -> 0.44.
+// ms, 26 (edge factor 16) 7.64 -> 6.68, 24 1.70 -> 1.37, 22 with 2^27 edges
+// 0.86 -> 0.59.
 //
 // A bucket is one word of up to four fields; a field holds the identifying
 // bits of one vertex and, in its top bit, whether this block knows the vertex
@@ -311,8 +312,11 @@ __global__ void __launch_bounds__(512, Q >= 4 ? (kZ ? 1 : 2) : (kZ ? 2 : (kDirec
 // Empty fields hold bits of a vertex of the same bucket (or of none below n)
 // and no flag, so they cannot answer wrongly.
 //
-// Flags are learnt in bulk: after its 1st, 2nd, 4th, 8th ... claim a warp
-// looks up its share of the table's vertices. Learning inside the loop, for
+// Flags are learnt in bulk: after its 2nd, 8th, 32nd ... claim a warp looks up
+// its share of the table's vertices. A round costs up to 98K lookups a block,
+// most of a claim's: R-MAT scale 24 takes 1.42 ms with rounds after the 1st,
+// 2nd, 4th, 8th ... claim, 1.37 after the 1st, 4th, 16th ..., 1.35 like this and
+// 1.36 after the 4th, 16th, 64th. Learning inside the loop, for
 // every lookup that found 0, cost more instructions than the table saved
 // requests (1.74 ms on R-MAT scale 24); only the queue form does it, and only
 // during its first claim, when the hubs have just joined and their lookups
@@ -341,18 +345,10 @@ __global__ void __launch_bounds__(kHubBlock, 1)
   const RootR fn = RootR::load(ctrl);
   uint32_t *const S = slots<RootR>(P);
   const uint64_t pol = policy_evict_first();
-  uint32_t *const H = ring_smem;
-  for (uint32_t i = threadIdx.x; i < kWideBuckets / 4; i += kHubBlock)
-    reinterpret_cast<uint4 *>(H)[i] = __ldg(reinterpret_cast<const uint4 *>(wide) + i);
+  WideTable table;
+  table.load(ring_smem, wide, s_bits, ways);
   WarpRing ring;
   ring.init(ring_smem + kWideBuckets, nullptr, nullptr, kNeverDirect);
-  const uint32_t fbits = s_bits - kWideBits + 1u;  // field width: identifying bits and flag
-  const uint32_t flag = 1u << (fbits - 1u), rmask = flag - 1u;
-  uint32_t ones = 0;
-  for (uint32_t w = 0; w < ways; ++w) ones |= 1u << (w * fbits);
-  const uint32_t highs = ones * flag;
-  const uint32_t down = 32u - s_bits;
-  const uint32_t mul = kWideMul << down;  // the product's s bits at the top of the word
   __syncthreads();
   const uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
   if (t == 0 && head) single_edge(P, fn, head, n, ctrl);
@@ -363,10 +359,6 @@ __global__ void __launch_bounds__(kHubBlock, 1)
       const uint64_t q = base + (uint64_t)j * 32u;
       e[j] = q < n_quads ? ld_edges_now(e4 + q, pol) : make_uint4(0u, 0u, 0u, 0u);
     }
-  };
-  // The flag bits of the fields of bucket word `word` that hold y's vertex.
-  auto holds = [&](uint32_t word, uint32_t y) {
-    return ~(((word ^ (((y >> down) & rmask) * ones)) | highs) - ones) & highs;
   };
   // kZ: joins `count` queued edges (ids; top bit: known to be in the tree of name 0).
   auto resolve = [&](uint32_t count) {
@@ -406,9 +398,7 @@ __global__ void __launch_bounds__(kHubBlock, 1)
     }
 #pragma unroll
     for (int i = 0; i < 4 * Q; ++i) {
-      const uint32_t y = x[i] * mul;
-      const uint32_t word = H[y >> (32u - kWideBits)];
-      const bool known = (holds(word, y) & word) != 0u;
+      const bool known = table.known(x[i]);
       if (kZ) {
         p[i] = 0xFFFFFFFFu;
         if (!known) p[i] = ldP(Z + (fn.f(x[i]) >> 5));
@@ -419,11 +409,8 @@ __global__ void __launch_bounds__(kHubBlock, 1)
     }
     if (!kZ && learning) {
 #pragma unroll
-      for (int i = 0; i < 4 * Q; ++i) {
-        const uint32_t y = x[i] * mul;
-        const uint32_t word = H[y >> (32u - kWideBits)], found = holds(word, y) & ~word;
-        if (p[i] == 0u && found) atomicOr(H + (y >> (32u - kWideBits)), found);
-      }
+      for (int i = 0; i < 4 * Q; ++i)
+        if (p[i] == 0u) table.learn(x[i]);
     }
 #pragma unroll
     for (int k = 0; k < 2 * Q; ++k) {
@@ -447,7 +434,7 @@ __global__ void __launch_bounds__(kHubBlock, 1)
   };
   constexpr uint32_t kGrab = kHubClaimQuads / (32u * Q);
   const uint32_t steps = (uint32_t)((n_quads + 32u * Q - 1) / (32u * Q));  // below 2^32 (kHubMaxQuads)
-  for (uint32_t claims = 0;;) {
+  for (uint32_t claims = 0, learn_at = 2;;) {
     uint32_t g0 = 0;
     if (ring.lane == 0) g0 = (uint32_t)min(atomicAdd(work, (unsigned long long)kGrab), (unsigned long long)steps);
     g0 = __shfl_sync(0xFFFFFFFFu, g0, 0);
@@ -467,20 +454,10 @@ __global__ void __launch_bounds__(kHubBlock, 1)
       step(cur, claims == 0u);
     }
     ++claims;
-    if ((claims & (claims - 1u)) == 0u) {
-      constexpr uint32_t kShare = kWideBuckets / (kHubBlock / 32);
-      const uint32_t b0 = (threadIdx.x >> 5) * kShare;
-      for (uint32_t b = b0 + ring.lane; b < b0 + kShare; b += 32u) {
-        const uint32_t word = H[b];
-        uint32_t found = 0u;
-        for (uint32_t w = 0; w < ways; ++w) {
-          const uint32_t f = word >> (w * fbits);
-          const uint32_t v = (((b << (s_bits - kWideBits)) | (f & rmask)) * kWideInv) & (0xFFFFFFFFu >> down);
-          if ((f & flag) || v >= n) continue;
-          if (kZ ? zbit(Z, fn.f(v)) : ldP_cg(P + v) == 0u) found |= flag << (w * fbits);
-        }
-        if (found) atomicOr(H + b, found);
-      }
+    if (claims == learn_at) {
+      learn_at *= 4;
+      table.learn_share<kHubBlock / 32>(
+          n, [&](uint32_t v) { return kZ ? zbit(Z, fn.f(v)) : ldP_cg(P + v) == 0u; });
     }
   }
   if (kZ) {
@@ -912,9 +889,7 @@ constexpr uint64_t kMinWaves = 8;
 // The queue form reads P through L2 only from this many vertices up (16 MB).
 constexpr uint32_t kL2MinVertices = 1u << 22;
 
-// The wide hot-vertex table pays from about 2^23 edges up: copying it costs a
-// block 128 KB, and below that a warp has at most one claim to learn from.
-constexpr uint64_t kHubMinQuads = 1ULL << 22, kHubMaxQuads = 1ULL << 37;
+constexpr uint64_t kHubMaxQuads = 1ULL << 37;
 
 // Claim size of the dynamic schedule, in warp steps. From 2^20 edges up,
 // 16 steps at a time (measured best there: fewer warps start on the hub's
@@ -962,8 +937,7 @@ cudaError_t edge_pass_q(int filter, int block, const EdgeSpan &e, uint32_t *P, u
     // the certificate word chooses among the launched instances (see
     // k_edge_pass_filtered); zsel: with Z, hub: without it
     const uint32_t *wsel = Z ? zsel : hub;
-    if (F::kRF && wide_hot && wsel && work && !log && !skip && !one_shot && e.n_quads >= kHubMinQuads &&
-        e.n_quads < kHubMaxQuads) {
+    if (F::kRF && wide_hot && wsel && work && !log && !skip && !one_shot && e.n_quads < kHubMaxQuads) {
       const uint32_t sb = id_bits(n);
       const void *k = Z ? (const void *)k_edge_pass_hub<true> : (const void *)k_edge_pass_hub<false>;
       static std::atomic<unsigned long long> set_z{0}, set_p{0};
