@@ -145,8 +145,8 @@ def measured_peaks():
 def kernel_source_sha() -> str:
     """Hash of the code that sets the edge pass's traffic: csrc/cc_device.cuh,
     the root selection (csrc/cc_rootsel.cu and csrc/cc_internal.h: its sample
-    fills the hot-vertex table the pass reads), and the text of the
-    k_edge_pass_filtered definition and of grab_for in csrc/cc_kernels.cu
+    fills the hot-vertex tables the pass reads), and the text of the
+    k_edge_pass_filtered and k_edge_pass_hub definitions and of grab_for in csrc/cc_kernels.cu
     (other host launch code in that file does not change the traffic)."""
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2507_03695_gb300", "csrc")
@@ -155,20 +155,21 @@ def kernel_source_sha() -> str:
             h.update(f.read())
     with open(os.path.join(csrc, "cc_kernels.cu")) as f:
         text = f.read()
-    start = text.index("k_edge_pass_filtered(const uint4")  # the definition, not a launch
-    start = text.rindex("template", 0, start)
     grab = text.index("uint32_t grab_for(")  # the dynamic schedule's claim size
     h.update(text[grab:text.index("\n}\n", grab)].encode())
-    depth, i = 0, text.index("{", start)
-    while True:
-        if text[i] == "{":
-            depth += 1
-        elif text[i] == "}":
-            depth -= 1
-            if depth == 0:
-                break
-        i += 1
-    h.update(text[start:i + 1].encode())
+    for name in ("k_edge_pass_filtered", "k_edge_pass_hub"):
+        start = text.index(name + "(const uint4")  # the definition, not a launch
+        start = text.rindex("template", 0, start)
+        depth, i = 0, text.index("{", start)
+        while True:
+            if text[i] == "{":
+                depth += 1
+            elif text[i] == "}":
+                depth -= 1
+                if depth == 0:
+                    break
+            i += 1
+        h.update(text[start:i + 1].encode())
     return h.hexdigest()[:16]
 
 
@@ -399,7 +400,7 @@ def edge_pass_roofline(graphs, phase_ms, workload: str, names, peak: float, peak
             "traffic": sum(traffic.values()) / len(traffic) if traffic else None,
             "traffic_by_graph": traffic,
             "algorithmic_bytes_per_launch": sum(edge_bytes) / len(edge_bytes),
-            "kernel": "edge pass (k_edge_pass_filtered), one launch per graph per step; achieved, traffic and "
+            "kernel": "edge pass (k_edge_pass_hub on R-MAT graphs, k_edge_pass_filtered on grids), one launch per graph per step; achieved, traffic and "
                       "algorithmic bytes are means over those launches",
             "peak_source": f"{peak_kind} (HBM copy bandwidth, MEASURED_PEAKS.json hbm_gbs)",
             "algorithmic_bytes": "8 B per edge per launch"}
