@@ -1009,7 +1009,7 @@ def bench_batched(args, cc, graphgen, torch, stream):
             "ms_p99": percentile(lat, 99), "runs": reps, "tuned_config": best, "tuner": tuner,
             "plain_gteps": E / (pmed * 1e-3) / 1e9, "plain_ms_p50": pmed, "plain_ms_p99": percentile(plain_ms, 99),
             "speedup_vs_plain": pmed / med, "labels_equal_plain": same,
-            "launch": "one cooperative persistent kernel, replayed from a CUDA graph",
+            "launch": "one sequence of launches for all graphs, replayed from a CUDA graph",
             "roofline": {"bound": "hbm", "achieved": alg / (med * 1e-3) / 1e9, "peak": peak, "unit": "GB/s",
                          "frac": alg / (med * 1e-3) / 1e9 / peak, "traffic": None,
                          "algorithmic_bytes_per_launch": alg,
