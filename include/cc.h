@@ -198,7 +198,9 @@ CC_API cc_status cc_run_csr(cc_graph *g, const uint64_t *offsets_dev, const uint
  * first chunk (the sampled leader when a hub shows, else the first chunk's
  * argmax) while the certificate's or the histogram's counts accumulate, then
  * one more init + edge pass only if m' was not the exact m; with sampled
- * selection, nothing until the last chunk. The labels go to L_out_host
+ * selection, nothing until the last chunk. A small graph (at most 1,572,864
+ * vertices, one chunk) is copied whole and then runs as cc_run does. The
+ * labels go to L_out_host
  * (uint32[n_vertices], may be NULL). Synchronising: returns after the labels
  * are in host memory, with any device error. */
 CC_API cc_status cc_run_host(cc_graph *g, const uint32_t *edges_host, uint64_t n_edges,
