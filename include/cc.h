@@ -171,7 +171,9 @@ CC_API cc_status cc_create(uint64_t n_vertices, uint64_t n_edges_capacity, const
  * edge count of its size class (below or from 2^31 edges); after that, a call
  * with the same buffers enqueues only stream work (kernels and memsets) and
  * can be captured into a CUDA graph. Each replay reads the captured edge
- * buffer as it is at replay time and rewrites P and the labels. */
+ * buffer as it is at replay time and rewrites P and the labels. With
+ * hbm_budget_bytes set, a captured run leaves out the scratch that a later
+ * buffer may displace, and takes the passes that need none. */
 CC_API cc_status cc_run(cc_graph *g, const uint32_t *edges_dev, uint64_t n_edges, uint32_t *L_out_dev,
                  cc_stream_t stream);
 

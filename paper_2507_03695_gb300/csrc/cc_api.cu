@@ -158,7 +158,8 @@ void dev_free(cc_graph *g, void *p, size_t bytes) {
 }
 
 // Scratch that only speeds a run up: the passes that use it fall back to the
-// general ones without it.
+// general ones without it. It may be freed for a needed buffer under a budget,
+// so nothing that outlives the call may name it (may_use_optional).
 void free_optional(cc_graph *g) {
   dev_free(g, g->wide_hot, sizeof(cc::WideHot));
   dev_free(g, g->bits, cc::bits_bytes(g->n));
@@ -185,6 +186,15 @@ void optional_alloc(cc_graph *g, void **p, size_t bytes) {
     *p = nullptr;
     cudaGetLastError();  // not an error of the call
   }
+}
+
+// Whether a run on s may use the optional scratch. A captured run may be
+// replayed after the scratch has been freed, which only a budget can cause: on
+// such a handle a captured run takes the general passes.
+bool may_use_optional(const cc_graph *g, cudaStream_t s) {
+  if (!g->opt.hbm_budget_bytes || (!g->bits && !g->wide_hot)) return true;
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(s, &st) == cudaSuccess && st == cudaStreamCaptureStatusNone;
 }
 
 size_t p_bytes(uint64_t n) { return (size_t)((n + 3) / 4 * 4) * sizeof(uint32_t); }
@@ -231,7 +241,7 @@ uint32_t select_stride(const cc_graph *g) {
 }
 
 cc_status root_select(cc_graph *g, const uint32_t *edges, uint64_t n_edges, const cc::EdgeSpan &span,
-                      cudaStream_t s, int *m_src) {
+                      cudaStream_t s, int *m_src, bool optional) {
   const uint32_t n = (uint32_t)g->n;
   const uint32_t stride = select_stride(g);
   const bool sampled = stride > 1;
@@ -248,7 +258,7 @@ cc_status root_select(cc_graph *g, const uint32_t *edges, uint64_t n_edges, cons
     return CC_OK;
   }
   CC_TRY(cc::launch_root_select_certified(edges, n_edges, span, g->cnt, wide, n, g->cert, g->ctrl, s, g->push,
-                                         g->push_cap, g->cand_list, g->cand_cap, wide_hot_for(g, n_edges)));
+                                         g->push_cap, g->cand_list, g->cand_cap, optional ? wide_hot_for(g, n_edges) : nullptr));
   return CC_OK;
 }
 
@@ -451,6 +461,7 @@ cc_status cc_run(cc_graph *g, const uint32_t *edges_dev, uint64_t n_edges, uint3
     g->ncomp_fresh = true;
     return CC_OK;
   }
+  const bool optional = may_use_optional(g, s);
   begin_timed_run(g);
   record(g, 0, s);
   int m_src = cc::kMFromHint;
@@ -459,7 +470,7 @@ cc_status cc_run(cc_graph *g, const uint32_t *edges_dev, uint64_t n_edges, uint3
     if (g->opt.root_hint != CC_ROOT_AUTO) {
       hint = (uint32_t)g->opt.root_hint;
     } else {
-      cc_status st = root_select(g, edges_dev, n_edges, span, s, &m_src);
+      cc_status st = root_select(g, edges_dev, n_edges, span, s, &m_src, optional);
       if (st != CC_OK) return st;
     }
   }
@@ -474,12 +485,12 @@ cc_status cc_run(cc_graph *g, const uint32_t *edges_dev, uint64_t n_edges, uint3
   uint32_t *Z = (g->z && (g->z_forced || exact)) ? g->z : nullptr;
   const uint32_t *zsel = (Z && !g->z_forced) ? &g->ctrl->cert : nullptr;
   record(g, 2, s);
-  if (g->bits && cc::bits_pass_fits(n, n_edges)) {
+  if (optional && g->bits && cc::bits_pass_fits(n, n_edges)) {
     CC_TRY(cc::launch_edge_pass_bits(g->rf, span, g->P, n, g->ctrl, g->bits, s));
   } else {
     CC_TRY(cc::launch_edge_pass(g->rf, eff_filter(g), eff_ept(g), eff_block(g), span, g->P, n, g->ctrl,
                                 nullptr, s, Z, zsel, false, nullptr, exact ? &g->ctrl->cert : nullptr, true,
-                                exact ? g->cert->hot : nullptr, exact ? wide_hot_for(g, n_edges) : nullptr));
+                                exact ? g->cert->hot : nullptr, exact && optional ? wide_hot_for(g, n_edges) : nullptr));
   }
   record(g, 3, s);
   CC_TRY(cc::launch_flatten(g->rf, g->opt.label_space, g->P, n, L_out_dev, g->ctrl, s));
@@ -600,7 +611,7 @@ static cc_status run_host_impl(cc_graph *g, const void *edges_host, uint64_t n_e
       CC_TRY(cudaStreamWaitEvent(s, g->copy_ev, 0));
     }
     int m_src = cc::kMFromHint;
-    cc_status st = root_select(g, g->staging, n_edges, all, s, &m_src);
+    cc_status st = root_select(g, g->staging, n_edges, all, s, &m_src, false);
     if (st != CC_OK) return st;
     CC_TRY(cc::launch_init(g->rf, g->P, n, g->ctrl, m_src, hint, s));
     CC_TRY(cc::launch_edge_pass(g->rf, eff_filter(g), eff_ept(g), eff_block(g), all, g->P, n, g->ctrl,
