@@ -84,7 +84,9 @@ typedef struct cc_server_config {
   uint64_t hbm_budget_bytes;       /* device arena for resident graphs (required)   */
   uint32_t max_graphs;             /* graph ids 0 .. max_graphs-1; 0 = 1024          */
   uint32_t executor_blocks_per_sm; /* resident executor blocks (256 threads); 0 = 3, which
-                                      leaves room on every SM for the side-stream kernels */
+                                      leaves room on every SM for the side-stream kernels and
+                                      for the calls of cc.h; with more, exact-selection runs
+                                      of cc.h wait until the executor leaves */
   uint32_t tile_edges;             /* largest executor tile in edges or pairs; 0 = 16384;
                                       requests are cut finer to spread over all blocks */
   uint32_t idle_timeout_us;        /* executor leaves after this much idleness; 0 = 20000 */

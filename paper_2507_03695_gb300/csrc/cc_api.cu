@@ -159,7 +159,7 @@ void dev_free(cc_graph *g, void *p, size_t bytes) {
 
 // Scratch that only speeds a run up: the passes that use it fall back to the
 // general ones without it. It may be freed for a needed buffer under a budget,
-// so nothing that outlives the call may name it (may_use_optional).
+// so nothing that outlives the call may name it (passes_for).
 void free_optional(cc_graph *g) {
   dev_free(g, g->wide_hot, sizeof(cc::WideHot));
   dev_free(g, g->bits, cc::bits_bytes(g->n));
@@ -188,13 +188,30 @@ void optional_alloc(cc_graph *g, void **p, size_t bytes) {
   }
 }
 
-// Whether a run on s may use the optional scratch. A captured run may be
-// replayed after the scratch has been freed, which only a budget can cause: on
-// such a handle a captured run takes the general passes.
-bool may_use_optional(const cc_graph *g, cudaStream_t s) {
-  if (!g->opt.hbm_budget_bytes || (!g->bits && !g->wide_hot)) return true;
-  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-  return cudaStreamIsCapturing(s, &st) == cudaSuccess && st == cudaStreamCaptureStatusNone;
+// The passes of cc_run that take more than the general one does.
+struct Passes {
+  bool one_block, bits, wide;
+};
+
+// A captured run may be replayed after optional scratch has been freed, which
+// only a budget can cause, and while a server is open: on a handle with a budget
+// it names no such scratch, and it never takes the pass that waits for the
+// serving executor to leave. (With the bitmap the other form waits as well.)
+Passes passes_for(const cc_graph *g, uint64_t n_edges, cudaStream_t s, uint32_t executor_blocks) {
+  const bool room = executor_blocks <= (uint32_t)cc::kExecutorDefault;
+  Passes p;
+  p.one_block = g->bits && room && !g->opt.timing && cc::tiny_fits(g->n, n_edges);  // (timed runs keep their phases apart)
+  p.bits = g->bits && room && cc::bits_pass_fits(g->n, n_edges);
+  p.wide = wide_hot_for(g, n_edges) && (g->z || executor_blocks == 0);
+  const bool budget = g->opt.hbm_budget_bytes != 0;
+  if ((budget && (p.bits || p.wide)) || (p.wide && !g->z)) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) {
+      p.bits = p.bits && !budget;
+      p.wide = p.wide && g->z && !budget;
+    }
+  }
+  return p;
 }
 
 size_t p_bytes(uint64_t n) { return (size_t)((n + 3) / 4 * 4) * sizeof(uint32_t); }
@@ -241,7 +258,7 @@ uint32_t select_stride(const cc_graph *g) {
 }
 
 cc_status root_select(cc_graph *g, const uint32_t *edges, uint64_t n_edges, const cc::EdgeSpan &span,
-                      cudaStream_t s, int *m_src, bool optional) {
+                      cudaStream_t s, int *m_src, bool wide_table) {
   const uint32_t n = (uint32_t)g->n;
   const uint32_t stride = select_stride(g);
   const bool sampled = stride > 1;
@@ -258,7 +275,7 @@ cc_status root_select(cc_graph *g, const uint32_t *edges, uint64_t n_edges, cons
     return CC_OK;
   }
   CC_TRY(cc::launch_root_select_certified(edges, n_edges, span, g->cnt, wide, n, g->cert, g->ctrl, s, g->push,
-                                         g->push_cap, g->cand_list, g->cand_cap, optional ? wide_hot_for(g, n_edges) : nullptr));
+                                         g->push_cap, g->cand_list, g->cand_cap, wide_table ? wide_hot_for(g, n_edges) : nullptr));
   return CC_OK;
 }
 
@@ -451,7 +468,9 @@ cc_status cc_run(cc_graph *g, const uint32_t *edges_dev, uint64_t n_edges, uint3
   g->applied = n_edges;
   const uint32_t n = (uint32_t)g->n;
   const cc::EdgeSpan span = cc::split_edges(edges_dev, n_edges);
-  if (g->bits && !g->opt.timing && cc::tiny_fits(n, n_edges)) {  // (timed runs keep their phases apart)
+  const cc::ExecutorBlocks executor(g->device);
+  const Passes take = passes_for(g, n_edges, s, executor.count());
+  if (take.one_block) {
     const bool select = g->rf && g->opt.root_hint == CC_ROOT_AUTO;
     const uint32_t hint = g->rf && !select ? (uint32_t)g->opt.root_hint : 0u;
     CC_TRY(cc::launch_tiny(g->rf, span, g->P, n, g->ctrl, select ? select_stride(g) : 0u, hint, g->opt.label_space,
@@ -461,7 +480,6 @@ cc_status cc_run(cc_graph *g, const uint32_t *edges_dev, uint64_t n_edges, uint3
     g->ncomp_fresh = true;
     return CC_OK;
   }
-  const bool optional = may_use_optional(g, s);
   begin_timed_run(g);
   record(g, 0, s);
   int m_src = cc::kMFromHint;
@@ -470,7 +488,7 @@ cc_status cc_run(cc_graph *g, const uint32_t *edges_dev, uint64_t n_edges, uint3
     if (g->opt.root_hint != CC_ROOT_AUTO) {
       hint = (uint32_t)g->opt.root_hint;
     } else {
-      cc_status st = root_select(g, edges_dev, n_edges, span, s, &m_src, optional);
+      cc_status st = root_select(g, edges_dev, n_edges, span, s, &m_src, take.wide);
       if (st != CC_OK) return st;
     }
   }
@@ -485,12 +503,12 @@ cc_status cc_run(cc_graph *g, const uint32_t *edges_dev, uint64_t n_edges, uint3
   uint32_t *Z = (g->z && (g->z_forced || exact)) ? g->z : nullptr;
   const uint32_t *zsel = (Z && !g->z_forced) ? &g->ctrl->cert : nullptr;
   record(g, 2, s);
-  if (optional && g->bits && cc::bits_pass_fits(n, n_edges)) {
+  if (take.bits) {
     CC_TRY(cc::launch_edge_pass_bits(g->rf, span, g->P, n, g->ctrl, g->bits, s));
   } else {
     CC_TRY(cc::launch_edge_pass(g->rf, eff_filter(g), eff_ept(g), eff_block(g), span, g->P, n, g->ctrl,
                                 nullptr, s, Z, zsel, false, nullptr, exact ? &g->ctrl->cert : nullptr, true,
-                                exact ? g->cert->hot : nullptr, exact && optional ? wide_hot_for(g, n_edges) : nullptr));
+                                exact ? g->cert->hot : nullptr, exact && take.wide ? wide_hot_for(g, n_edges) : nullptr));
   }
   record(g, 3, s);
   CC_TRY(cc::launch_flatten(g->rf, g->opt.label_space, g->P, n, L_out_dev, g->ctrl, s));

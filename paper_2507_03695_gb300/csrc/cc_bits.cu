@@ -40,10 +40,12 @@ namespace cc {
 namespace {
 
 constexpr uint32_t kChunkQuads = 64;  // 128 edges, four per lane of a warp
-constexpr int kFilterBlock = 1024;
+constexpr int kFilterBlock = 512;
 constexpr int kLinkBlock = 256;
 constexpr size_t kFilterQueueBytes = (kFilterBlock / 32) * 2 * kRing * sizeof(uint32_t);
-static_assert(kBitsVertices / 8 + kFilterQueueBytes <= 224 * 1024, "the bits and the queues fit a block's shared memory");
+static_assert(kBitsVertices / 8 + kFilterQueueBytes <= kBesideExecutorSmem, "the bits and the queues fit beside the executor");
+// Two blocks on an SM where their bits fit.
+constexpr size_t kFilterPairBytes = kSmemPerSM / 2 - kSmemPerBlock;
 
 // One linking round over the chunks k * stride + first. kFirst: P holds every
 // vertex's own name, so the endpoints need no parent loads.
@@ -118,7 +120,10 @@ __global__ void __launch_bounds__(256) k_bits_build(const uint4 *__restrict__ e4
     const uint32_t ref = __shfl_sync(0xFFFFFFFFu, r, (int)best);
     if (lane == 0) {
       s_ref = ref;
-      if (blockIdx.x == 0) ctrl->ref = ref;
+      if (blockIdx.x == 0) {
+        ctrl->ref = ref;
+        ctrl->work = 0ULL;  // step 3's claims
+      }
     }
   }
   if (kBits) __syncthreads();
@@ -167,12 +172,17 @@ __global__ void __launch_bounds__(256) k_bits_build(const uint4 *__restrict__ e4
   }
 }
 
-// Step 3. One block of 32 warps per SM; a warp's next chunk is loaded while it
-// works on one.
+// Step 3. Blocks of 16 warps, because one of 32 would not fit beside the serving
+// executor's; a warp's next chunk is loaded while it works on one. Long lists are
+// claimed kGrab chunks at a time: with a fixed split into one block per SM the
+// pass took either 235 or 550 us on R-MAT scale 20 with 2^26 edges, from run to
+// run. Whole calls with one static block of 32 warps and like this, us: R-MAT scale
+// 16 (f = id) 85 and 86, 18 (f = id) 111 and 107, 19 206 and 196, 20 with 2^26
+// edges 538 and 502, 1,000,003 vertices with 16M edges 270 and 275.
 template <class F>
-__global__ void __launch_bounds__(kFilterBlock, 1)
+__global__ void __maxnreg__(kBesideExecutorRegs / kFilterBlock)
     k_bits_filter(const uint4 *__restrict__ e4, uint64_t n_quads, const uint2 *head, const uint2 *tail, uint32_t *P,
-                  uint32_t n, Ctrl *ctrl, const uint32_t *__restrict__ all_bits) {
+                  uint32_t n, Ctrl *ctrl, const uint32_t *__restrict__ all_bits, uint32_t grab) {
   extern __shared__ uint32_t smem[];
   const F fn = F::load(ctrl);
   uint32_t *const S = slots<F>(P);
@@ -208,8 +218,20 @@ __global__ void __launch_bounds__(kFilterBlock, 1)
   };
   const uint64_t pol = policy_evict_first();
   const uint64_t chunks = (n_quads + kChunkQuads - 1) / kChunkQuads, full = n_quads / kChunkQuads;
+  // grab > 1: chunks [ch, end) are claimed from a counter, and the claim after
+  // them is asked for when they begin; else a fixed stride of chunks
   const uint64_t hop = (uint64_t)gridDim.x * (kFilterBlock / 32);
-  uint64_t ch = (uint64_t)wid * gridDim.x + blockIdx.x;
+  unsigned long long next = 0;
+  uint64_t ch = (uint64_t)wid * gridDim.x + blockIdx.x, end = ch + 1;
+  auto claim = [&]() {
+    ch = __shfl_sync(0xFFFFFFFFu, next, 0);
+    end = ch + grab;
+    if (lane == 0) next = atomicAdd(&ctrl->work, (unsigned long long)grab);
+  };
+  if (grab > 1u) {
+    if (lane == 0) next = atomicAdd(&ctrl->work, (unsigned long long)grab);
+    claim();
+  }
   uint4 e[2];
   auto load = [&]() {
     const uint4 *const p = e4 + ch * kChunkQuads + lane;
@@ -225,7 +247,14 @@ __global__ void __launch_bounds__(kFilterBlock, 1)
   if (ch < chunks) load();
   while (ch < chunks) {
     uint32_t x[8] = {e[0].x, e[0].y, e[0].z, e[0].w, e[1].x, e[1].y, e[1].z, e[1].w};
-    ch += hop;
+    if (++ch == end) {
+      if (grab > 1u) {
+        claim();
+      } else {
+        ch += hop - 1u;
+        end = ch + 1u;
+      }
+    }
     if (ch < chunks) load();
     const uint32_t top = max(max(max(x[0], x[1]), max(x[2], x[3])), max(max(x[4], x[5]), max(x[6], x[7])));
     if (top >= n) {
@@ -264,6 +293,7 @@ __global__ void __launch_bounds__(kFilterBlock, 1)
 constexpr int kRounds = 4;
 constexpr uint64_t kFirstSample = 2, kShrink = 4;
 constexpr uint64_t kMinSampleChunks = 32;
+constexpr uint32_t kGrab = 8;
 
 template <class F>
 cudaError_t bits_pass(const EdgeSpan &e, uint32_t *P, uint32_t n, Ctrl *ctrl, uint32_t *bits, cudaStream_t s) {
@@ -292,9 +322,11 @@ cudaError_t bits_pass(const EdgeSpan &e, uint32_t *P, uint32_t n, Ctrl *ctrl, ui
   const cudaError_t err = ensure_func_attr(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)(kBitsVertices / 8 + kFilterQueueBytes), smem_set);
   if (err != cudaSuccess) return err;
-  const unsigned gf = clamp_grid((chunks + kFilterBlock / 32 - 1) / (kFilterBlock / 32), (uint64_t)num_sms());
-  k_bits_filter<F><<<gf, kFilterBlock, bits_bytes(n) + kFilterQueueBytes, s>>>(e.quads, e.n_quads, e.head, e.tail, P, n,
-                                                                             ctrl, bits);
+  const size_t smem = bits_bytes(n) + kFilterQueueBytes;
+  const unsigned gf = clamp_grid((chunks + kFilterBlock / 32 - 1) / (kFilterBlock / 32),
+                                 (uint64_t)num_sms() * (smem <= kFilterPairBytes ? 2u : 1u));
+  const uint32_t grab = chunks >= (uint64_t)gf * (kFilterBlock / 32) * 4u * kGrab ? kGrab : 1u;
+  k_bits_filter<F><<<gf, kFilterBlock, smem, s>>>(e.quads, e.n_quads, e.head, e.tail, P, n, ctrl, bits, grab);
   note_launch();
   return cudaGetLastError();
 }

@@ -70,6 +70,36 @@ inline unsigned clamp_grid(uint64_t want, uint64_t cap) {
   return (unsigned)(want < cap ? want : cap);
 }
 
+// What the serving executor leaves of an SM, at its default of 3 blocks: it holds
+// kExecutorBlock threads of kExecutorRegs registers and kExecutorSmem bytes a
+// block, and a block of another kernel that needs more than the rest waits until
+// it leaves, which under steady load it never does. So the kernels of the
+// single-graph calls stay within these bounds; the pass that cannot
+// (k_edge_pass_hub) is not launched while a server is open (ExecutorBlocks).
+constexpr int kExecutorBlock = 256, kExecutorRegs = 48, kExecutorDefault = 3;
+constexpr size_t kSmemPerSM = 228 << 10, kSmemPerBlock = 1 << 10;  // the second is taken by every block
+constexpr size_t kExecutorSmem = 8448;
+constexpr int kBesideExecutorRegs = 65536 - kExecutorDefault * kExecutorBlock * kExecutorRegs;
+constexpr size_t kBesideExecutorSmem =
+    kSmemPerSM - kExecutorDefault * (kExecutorSmem + kSmemPerBlock) - kSmemPerBlock;
+constexpr int kSmallBlockRegs = 32;  // blocks of 512 threads that fit beside four executor blocks
+
+// The most executor blocks per SM of the servers open on a device; 0: none is.
+// A server announces itself before it first launches an executor, and then waits
+// for the device, so that what was enqueued before cannot meet the executor. The
+// count holds while the object lives: a run is enqueued under it.
+class ExecutorBlocks {
+ public:
+  explicit ExecutorBlocks(int device);
+  ~ExecutorBlocks();
+  uint32_t count() const { return n_; }
+
+ private:
+  uint32_t n_;
+};
+void executor_announce(int device, uint32_t blocks_per_sm);
+void executor_withdraw(int device, uint32_t blocks_per_sm);
+
 // Sets a kernel attribute once per device. Setting a function attribute can
 // make the host wait for the device, so it is done on first use only, never
 // per launch; `done` is the call site's per-device bit mask.
@@ -308,12 +338,12 @@ bool tiny_fits(uint64_t n_vertices, uint64_t n_edges);
 cudaError_t launch_tiny(bool rf, const EdgeSpan &e, uint32_t *P, uint32_t n, Ctrl *ctrl, uint32_t count_stride,
                         uint32_t m_hint, int label_space, uint32_t *L, cudaStream_t s);
 // The edge pass by vertex bits in shared memory (cc_bits.cu), right after init:
-// graphs of at most kBitsVertices vertices (196,608 bytes of bits) and at
+// graphs of at most kBitsVertices vertices (195,584 bytes of bits) and at
 // least kBitsMinDegree edges per vertex (sparser ones have no giant component
 // to speak of: a grid's 1.8 edges per vertex took 1.3 times as long) and
 // kBitsMinEdges in all (below, its launches are most of the time).
 // bits: bits_bytes(n) bytes, 16-byte aligned.
-constexpr uint64_t kBitsVertices = 1536ULL << 10;
+constexpr uint64_t kBitsVertices = 1528ULL << 10;
 constexpr uint64_t kBitsMinEdges = 1ULL << 15, kBitsMaxEdges = 1ULL << 36, kBitsMinDegree = 3;
 constexpr size_t bits_bytes(uint64_t n) { return (size_t)((n + 127) / 128 * 16); }
 bool bits_pass_fits(uint64_t n_vertices, uint64_t n_edges);

@@ -9,9 +9,11 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <array>
 #include <atomic>
 #include <map>
 #include <mutex>
+#include <shared_mutex>
 
 #include "cc_device.cuh"
 #include "cc_internal.h"
@@ -293,7 +295,12 @@ __global__ void __launch_bounds__(512, Q >= 4 ? (kZ ? 1 : 2) : (kZ ? 2 : (kDirec
 
 // The edge pass of a certified hub on a large graph (from 2^22 vertices up,
 // default launch shape): as the hub forms above, with the wide hot-vertex
-// table (WideHot) in place of the 4096-entry one.
+// table (WideHot) in place of the 4096-entry one. Its blocks do not fit beside the
+// serving executor's, so without the bitmap it runs only while no server is
+// open (ExecutorBlocks) and in no captured run; the bitmap's other form (64 registers a thread, blocks
+// of 512) does not fit there either. Smaller blocks lose more than the table
+// gives: R-MAT scale 24, whole call, 1830 us with 1024 threads, 2274 with 512 of
+// 56 registers, 2395 with 576 of 48, 2500 with 704 of 40, 2176 without the table.
 //
 // What bounds it: the endpoint lookups, one L2 request each, at most 0.96 per
 // SM and clock; random shared-memory loads beside them cost nothing (16 per 8
@@ -492,37 +499,42 @@ __global__ void __launch_bounds__(256) k_validate(const uint4 *__restrict__ e4, 
   }
 }
 
-// A short insert in one block: every thread holds its pairs (at most 4) while
-// the block validates them, then hooks them. Four launches and two memsets
-// otherwise took longer than the work.
-constexpr int kInsertBlock = 1024;
-static_assert(kInsertOneBlock <= 4 * kInsertBlock, "four pairs per thread");
+// A short insert in one block, which validates all pairs, then hooks them, four
+// per thread at a time. Four launches and two memsets otherwise took longer than
+// the work.
+constexpr int kInsertBlock = 512;  // 1024 threads would not fit beside the serving executor
 
 template <class F>
-__global__ void __launch_bounds__(kInsertBlock) k_insert_small(const uint2 *__restrict__ e, uint32_t n_edges,
-                                                               uint32_t *P, uint32_t n, Ctrl *ctrl) {
+__global__ void __maxnreg__(kSmallBlockRegs) k_insert_small(const uint2 *__restrict__ e, uint32_t n_edges,
+                                                            uint32_t *P, uint32_t n, Ctrl *ctrl) {
   const F fn = F::load(ctrl);
   uint32_t *const S = slots<F>(P);
-  uint2 x[4];
   bool bad = false;
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const uint32_t i = threadIdx.x + (uint32_t)j * kInsertBlock;
-    x[j] = i < n_edges ? ld_edge(e + i) : make_uint2(0u, 0u);
-    bad |= x[j].x >= n || x[j].y >= n;
+#pragma unroll 4
+  for (uint32_t i = threadIdx.x; i < n_edges; i += kInsertBlock) {
+    const uint2 x = ld_edge(e + i);
+    bad |= x.x >= n || x.y >= n;
   }
   if (__syncthreads_or(bad)) {  // nothing is applied
     if (threadIdx.x == 0) set_err(ctrl, kErrRange);
     return;
   }
-  uint32_t p[8];
+  for (uint32_t i0 = threadIdx.x; i0 < n_edges; i0 += 4 * kInsertBlock) {
+    uint2 x[4];
+    uint32_t p[8];
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    p[2 * j] = ldP_cg(P + x[j].x);
-    p[2 * j + 1] = ldP_cg(P + x[j].y);
+    for (int j = 0; j < 4; ++j) {
+      const uint32_t i = i0 + (uint32_t)j * kInsertBlock;
+      x[j] = i < n_edges ? ld_edge(e + i) : make_uint2(0u, 0u);
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      p[2 * j] = ldP_cg(P + x[j].x);
+      p[2 * j + 1] = ldP_cg(P + x[j].y);
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) unite<true>(S, fn.f(x[j].x), p[2 * j], fn.f(x[j].y), p[2 * j + 1]);
   }
-#pragma unroll
-  for (int j = 0; j < 4; ++j) unite<true>(S, fn.f(x[j].x), p[2 * j], fn.f(x[j].y), p[2 * j + 1]);
 }
 
 // ------------------------------------------------------------------ flatten
@@ -816,6 +828,38 @@ std::atomic<unsigned long long> g_launches{0};
 
 void note_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 unsigned long long launch_count() { return g_launches.load(std::memory_order_relaxed); }
+
+namespace {
+struct Servers {
+  std::shared_mutex mu;
+  std::map<int, std::array<uint32_t, 9>> open;  // per device, servers by executor blocks per SM
+};
+Servers &servers() {
+  static Servers *s = new Servers();  // outlives every server
+  return *s;
+}
+}  // namespace
+
+ExecutorBlocks::ExecutorBlocks(int device) : n_(0) {
+  Servers &s = servers();
+  s.mu.lock_shared();
+  const auto it = s.open.find(device);
+  if (it != s.open.end())
+    for (uint32_t k = 1; k < it->second.size(); ++k)
+      if (it->second[k]) n_ = k;
+}
+ExecutorBlocks::~ExecutorBlocks() { servers().mu.unlock_shared(); }
+
+void executor_announce(int device, uint32_t blocks_per_sm) {
+  Servers &s = servers();
+  std::lock_guard<std::shared_mutex> lk(s.mu);
+  s.open[device][blocks_per_sm < 8 ? blocks_per_sm : 8]++;
+}
+void executor_withdraw(int device, uint32_t blocks_per_sm) {
+  Servers &s = servers();
+  std::lock_guard<std::shared_mutex> lk(s.mu);
+  s.open[device][blocks_per_sm < 8 ? blocks_per_sm : 8]--;
+}
 
 uint64_t persistent_cap(const void *kernel, int block, size_t smem) {
   struct Key {

@@ -269,10 +269,10 @@ __device__ __forceinline__ uint32_t bucket_of(uint32_t x) { return bucket_hash(x
 // ranks the owners and keeps the kCertTop best for the counting pass.
 // kList: the vertices are those appended to the list's segments (as many as
 // each segment holds), else every vertex 0 .. n-1.
-constexpr int kSelectBlock = 1024, kSelectBlocks = (int)kListSegs;  // the list form's launch
+constexpr int kSelectBlock = 512, kSelectBlocks = (int)kListSegs;  // the list form's launch
 
 template <bool kList>
-__global__ void __launch_bounds__(kList ? kSelectBlock : 256) k_select_candidates(const uint32_t *__restrict__ cnt, uint32_t n,
+__global__ void __maxnreg__(kSmallBlockRegs) k_select_candidates(const uint32_t *__restrict__ cnt, uint32_t n,
                                                            Ctrl *ctrl, CertScratch *cs,
                                                            const uint32_t *__restrict__ list, uint32_t list_cap,
                                                            WideHot *wide_hot, uint32_t s_bits, uint32_t ways, uint64_t sampled) {
@@ -475,11 +475,11 @@ struct CertCounter {
 
 // Every block clears and adds up all buckets, so a thread gets at least 16
 // edge loads. (Blocks of 1024 threads, half as many, would not fit beside the
-// serving executor's blocks.)
+// serving executor's blocks; see kBesideExecutorRegs.)
 constexpr int kCertBlock = 512;
 constexpr uint64_t kCertQuadsPerBlock = 16ull * kCertBlock;
 
-__global__ void __launch_bounds__(kCertBlock, 2)
+__global__ void __maxnreg__(kBesideExecutorRegs / kCertBlock)
     k_degree_certify(const uint4 *__restrict__ e4, uint64_t n_quads, const uint2 *head, const uint2 *tail, uint32_t n,
                      CertScratch *cs, Ctrl *ctrl, int decide, uint32_t *push_buf, uint32_t push_seg) {
   extern __shared__ uint32_t csm[];

@@ -166,12 +166,13 @@ constexpr int kEpt = 4;  // elements per thread per round
 // request's finished tiles. Blocks leave when the host sets `stop`, or when
 // a wait expires (exec_err tells the host). A gated apply tile waits at most
 // gate_ns for its request's validate tiles.
-__global__ void __launch_bounds__(256) k_executor(HostShared *hs, DevShared *ds, unsigned long long wait_ns,
+__global__ void __maxnreg__(kExecutorRegs) k_executor(HostShared *hs, DevShared *ds, unsigned long long wait_ns,
                                                   unsigned long long gate_ns) {
   __shared__ WorkItem it;
   __shared__ int s_leave;
   __shared__ unsigned int s_bad, s_skip;
-  __shared__ uint32_t ring_smem[8 * 4 * kRing];
+  __shared__ uint32_t ring_smem[kExecutorBlock / 32 * 4 * kRing];
+  static_assert(sizeof(ring_smem) + sizeof(WorkItem) + 16 <= kExecutorSmem, "room for other kernels");
   while (true) {
     if (threadIdx.x == 0) {
       int leave = 0;
@@ -521,6 +522,7 @@ struct cc_server {
   cudaStream_t exec_stream = nullptr, side_stream = nullptr;
   cudaStream_t side_streams[cc::srv::kSideStreams] = {};  // [0] is side_stream
   cudaEvent_t exec_ev = nullptr;
+  bool announced = false;  // to the single-graph calls (ExecutorBlocks)
   uint32_t *side_words = nullptr;  // pinned: per-graph m and error word read back after admission
   uint32_t *side_flags = nullptr;  // pinned: one rejection word per running side insert
   uint32_t *side_reject = nullptr; // device: the same words, written by validation
@@ -1076,7 +1078,7 @@ void manage_executor(cc_server *s) {
     s->idle_since = 0;
     if (!s->exec_running) {
       const unsigned grid = (unsigned)(cc::num_sms() * s->cfg.executor_blocks_per_sm);
-      cc::srv::k_executor<<<grid, 256, 0, s->exec_stream>>>(s->hs_dev, s->ds, s->wait_ns, s->gate_ns);
+      cc::srv::k_executor<<<grid, cc::kExecutorBlock, 0, s->exec_stream>>>(s->hs_dev, s->ds, s->wait_ns, s->gate_ns);
       cc::note_launch();
       cudaEventRecord(s->exec_ev, s->exec_stream);
       s->exec_running = true;
@@ -1216,6 +1218,7 @@ void scheduler_main(cc_server *s) {
 
 // Frees what cc_server_create allocated (any subset of it).
 void release_resources(cc_server *s) {
+  if (s->announced) cc::executor_withdraw(s->device, s->cfg.executor_blocks_per_sm);
   if (s->arena_base) cudaFree(s->arena_base);
   if (s->hs) cudaFreeHost(s->hs);
   if (s->ds) cudaFree(s->ds);
@@ -1293,7 +1296,7 @@ cudaError_t warm_up(cc_server *s) {
   // the executor: told to leave before it starts
   if (e == cudaSuccess) {
     *(volatile unsigned int *)&s->hs->stop = 1u;
-    cc::srv::k_executor<<<1, 256, 0, s->exec_stream>>>(s->hs_dev, s->ds, s->wait_ns, s->gate_ns);
+    cc::srv::k_executor<<<1, cc::kExecutorBlock, 0, s->exec_stream>>>(s->hs_dev, s->ds, s->wait_ns, s->gate_ns);
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->exec_stream);
     *(volatile unsigned int *)&s->hs->stop = 0u;
@@ -1324,7 +1327,7 @@ void cc_server_config_init(cc_server_config *cfg) {
   if (!cfg) return;
   memset(cfg, 0, sizeof(*cfg));
   cfg->max_graphs = 1024;
-  cfg->executor_blocks_per_sm = 3;
+  cfg->executor_blocks_per_sm = cc::kExecutorDefault;
   cfg->tile_edges = 16384;
   cfg->idle_timeout_us = 20000;
   cfg->mode = CC_ROOT_MAXDEG;
@@ -1336,7 +1339,7 @@ cc_status cc_server_create(const cc_server_config *cfg_in, cc_server **out) {
   *out = nullptr;
   cc_server_config cfg = *cfg_in;
   if (!cfg.max_graphs) cfg.max_graphs = 1024;
-  if (!cfg.executor_blocks_per_sm) cfg.executor_blocks_per_sm = 3;
+  if (!cfg.executor_blocks_per_sm) cfg.executor_blocks_per_sm = cc::kExecutorDefault;
   if (!cfg.tile_edges) cfg.tile_edges = 16384;
   if (!cfg.idle_timeout_us) cfg.idle_timeout_us = 20000;
   if (cfg.hbm_budget_bytes == 0 || cfg.executor_blocks_per_sm > 8 || cfg.tile_edges < 256 ||
@@ -1355,6 +1358,11 @@ cc_status cc_server_create(const cc_server_config *cfg_in, cc_server **out) {
   s->gate_ns = cfg.gate_wait_us ? (unsigned long long)cfg.gate_wait_us * 1000ULL : cc::srv::kGateTimeoutNs;
   s->hold_left = cfg.fault_hold_publish_us ? 1u : 0u;
   cudaError_t e = cudaGetDevice(&s->device);
+  if (e == cudaSuccess) {
+    cc::executor_announce(s->device, cfg.executor_blocks_per_sm);
+    s->announced = true;
+    e = cudaDeviceSynchronize();  // what was enqueued before may need whole SMs
+  }
   if (e == cudaSuccess) e = cudaMalloc((void **)&s->arena_base, cfg.hbm_budget_bytes);
   if (e == cudaSuccess) e = cudaHostAlloc((void **)&s->hs, sizeof(HostShared), cudaHostAllocMapped);
   if (e == cudaSuccess) e = cudaHostGetDevicePointer((void **)&s->hs_dev, s->hs, 0);

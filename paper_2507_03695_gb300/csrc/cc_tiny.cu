@@ -56,8 +56,12 @@ __device__ __forceinline__ void tiny_unite(uint32_t *p, const F fn, uint32_t a, 
 
 // count_stride: 0 no degree count (f = id, or m given); 1 all edges; k > 1 one
 // group of kSampleGroup edges in k.
+// (28,672 / 1024, in whole steps of 8 registers: it fits beside the serving executor)
+constexpr int kTinyRegs = kBesideExecutorRegs / kTinyBlock / 8 * 8;
+static_assert(kTinyVertices * sizeof(uint32_t) + 512 <= kBesideExecutorSmem, "and so do the parents");
+
 template <class F>
-__global__ void __launch_bounds__(kTinyBlock, 1)
+__global__ void __maxnreg__(kTinyRegs)
     k_tiny(const uint4 *__restrict__ e4, uint32_t n_quads, const uint2 *head, const uint2 *tail, uint32_t *P,
            uint32_t n, Ctrl *ctrl, uint32_t count_stride, uint32_t m_hint, int min_id, uint32_t *__restrict__ L) {
   extern __shared__ uint32_t p[];  // degrees, then parents

@@ -1,7 +1,8 @@
 """Captured runs on a handle with a memory budget: scratch that a later buffer
 of the handle may displace is not named by the captured launches, so a replay
 after such a call is sound. Without a budget nothing is displaced and a
-captured run takes the same passes as any other.
+captured run takes the same passes as any other, but for the wide hot-vertex
+table's.
 """
 import numpy as np
 import pytest
@@ -49,7 +50,8 @@ def test_replay_after_the_scratch_was_displaced(scale, repeats, mode):
     with cc.Graph(n, len(e), mode=mode) as g:
         fast = launches(g, d, L)
         graph, held = capture(g, d, L)
-        assert held == fast
+        # (the pass with the wide table waits for a server's executor: never captured)
+        assert held == (fast if repeats == 1 else general)
     # room for the scratch, or for the labels of a host run, not for both
     with cc.Graph(n, len(e), mode=mode, hbm_budget_bytes=least + 4 * n) as g:
         assert launches(g, d, L) == fast
