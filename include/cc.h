@@ -201,7 +201,7 @@ CC_API cc_status cc_run_csr(cc_graph *g, const uint64_t *offsets_dev, const uint
  * argmax) while the certificate's or the histogram's counts accumulate, then
  * one more init + edge pass only if m' was not the exact m; with sampled
  * selection, nothing until the last chunk. A small graph in one chunk (at most
- * 49,152 vertices and 32,767 edges; or at most 1,564,672 vertices with at least
+ * 49,152 vertices and 32,767 edges; or at most 1,540,096 vertices with at least
  * 32,768 edges and three edges per vertex) is copied whole and then runs as
  * cc_run does, unless the handle records phase times. The labels go to
  * L_out_host (uint32[n_vertices], may be NULL). Synchronising: returns after the labels

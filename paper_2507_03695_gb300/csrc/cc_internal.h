@@ -41,6 +41,8 @@ struct alignas(128) Ctrl {
   unsigned long long work;      // edge pass, dynamic schedule: steps claimed so far
   unsigned long long pairs;     // cc_forest_pairs: non-root vertices found
   uint32_t ref;                 // edge pass by bits: root name of the reference tree
+  uint32_t marked;              // edge pass by bits: the reference tree holds most sampled endpoints
+  uint32_t deep[4];             // edge pass by bits: linking round r has left deep trees
 };
 static_assert(offsetof(Ctrl, q_u) % 8 == 0, "the query pair is loaded with an 8-byte access");
 static_assert(offsetof(Ctrl, maxkey) % 8 == 0 && offsetof(Ctrl, ncomp) % 8 == 0, "64-bit atomics");
@@ -79,7 +81,11 @@ inline unsigned clamp_grid(uint64_t want, uint64_t cap) {
 constexpr int kExecutorBlock = 256, kExecutorRegs = 48, kExecutorDefault = 3;
 constexpr size_t kSmemPerSM = 228 << 10, kSmemPerBlock = 1 << 10;  // the second is taken by every block
 constexpr size_t kExecutorSmem = 8448;
+// Registers come in four parts with a quarter of the warps each.
 constexpr int kBesideExecutorRegs = 65536 - kExecutorDefault * kExecutorBlock * kExecutorRegs;
+constexpr bool beside_executor(int threads, int regs) {
+  return (threads / 32 + 3) / 4 * 32 * ((regs + 7) / 8 * 8) <= kBesideExecutorRegs / 4;
+}
 constexpr size_t kBesideExecutorSmem =
     kSmemPerSM - kExecutorDefault * (kExecutorSmem + kSmemPerBlock) - kSmemPerBlock;
 constexpr int kSmallBlockRegs = 32;  // blocks of 512 threads that fit beside four executor blocks
@@ -320,6 +326,9 @@ cudaError_t launch_edge_pass(bool rf, int filter, int ept, int block, const Edge
                              uint32_t *log = nullptr, const uint32_t *hub = nullptr, bool dyn = false,
                              const unsigned long long *hot = nullptr, const WideHot *wide_hot = nullptr,
                              bool settled = false);
+// The plain pass for any graph alone, its counter (ctrl->work) already zero.
+cudaError_t launch_edge_pass_general(bool rf, const EdgeSpan &e, uint32_t *P, uint32_t n, Ctrl *ctrl,
+                                     const uint32_t *skip, cudaStream_t s);
 // settled: the trees exist already, so the grid need not be kept small for the
 // edges that would all meet on the first roots.
 // An insert of at most kInsertOneBlock pairs: validation and hooking in one
@@ -338,12 +347,12 @@ bool tiny_fits(uint64_t n_vertices, uint64_t n_edges);
 cudaError_t launch_tiny(bool rf, const EdgeSpan &e, uint32_t *P, uint32_t n, Ctrl *ctrl, uint32_t count_stride,
                         uint32_t m_hint, int label_space, uint32_t *L, cudaStream_t s);
 // The edge pass by vertex bits in shared memory (cc_bits.cu), right after init:
-// graphs of at most kBitsVertices vertices (195,584 bytes of bits) and at
+// graphs of at most kBitsVertices vertices (192,512 bytes of bits) and at
 // least kBitsMinDegree edges per vertex (sparser ones have no giant component
 // to speak of: a grid's 1.8 edges per vertex took 1.3 times as long) and
 // kBitsMinEdges in all (below, its launches are most of the time).
 // bits: bits_bytes(n) bytes, 16-byte aligned.
-constexpr uint64_t kBitsVertices = 1528ULL << 10;
+constexpr uint64_t kBitsVertices = 1504ULL << 10;
 constexpr uint64_t kBitsMinEdges = 1ULL << 15, kBitsMaxEdges = 1ULL << 36, kBitsMinDegree = 3;
 constexpr size_t bits_bytes(uint64_t n) { return (size_t)((n + 127) / 128 * 16); }
 bool bits_pass_fits(uint64_t n_vertices, uint64_t n_edges);

@@ -1061,6 +1061,26 @@ cudaError_t launch_edge_pass(bool rf, int filter, int ept, int block, const Edge
                                   nullptr, nullptr, settled);
 }
 
+template <class F>
+cudaError_t edge_pass_general(const EdgeSpan &e, uint32_t *P, uint32_t n, Ctrl *ctrl, const uint32_t *skip,
+                              cudaStream_t s) {
+  constexpr int block = 512, Q = 2;
+  const size_t smem = (size_t)(block / 32) * 4 * kRing * sizeof(uint32_t);
+  const void *k = (const void *)k_edge_pass_filtered<F, Q, false, true>;
+  const uint64_t per = (uint64_t)block * Q * kMinWaves;
+  const unsigned g = clamp_grid((e.n_quads + per - 1) / per, persistent_cap(k, block, smem));
+  k_edge_pass_filtered<F, Q, false, true><<<g, block, smem, s>>>(e.quads, e.n_quads, e.head, e.tail, P, n, ctrl, skip,
+                                                                 nullptr, nullptr, nullptr, &ctrl->work,
+                                                                 grab_for(e.n_quads, Q, g, block), nullptr);
+  note_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t launch_edge_pass_general(bool rf, const EdgeSpan &e, uint32_t *P, uint32_t n, Ctrl *ctrl,
+                                     const uint32_t *skip, cudaStream_t s) {
+  return rf ? edge_pass_general<RootR>(e, P, n, ctrl, skip, s) : edge_pass_general<RootId>(e, P, n, ctrl, skip, s);
+}
+
 cudaError_t launch_validate(const EdgeSpan &e, uint32_t n, Ctrl *ctrl, cudaStream_t s, uint32_t *reject) {
   if (e.n_quads == 0 && !e.head && !e.tail) return cudaSuccess;
   const unsigned g = clamp_grid((e.n_quads + 255) / 256, persistent_cap((const void *)k_validate, 256, 0));

@@ -16,7 +16,7 @@ torch = pytest.importorskip("torch")
 cc = pytest.importorskip("paper_2507_03695_gb300")
 
 IDLE, LIMIT = 8.0, 2.0  # seconds
-MOST = 1528 << 10
+MOST = 1504 << 10
 HUB = (1 << 21) + 1, 65  # edges of the list, repeated on the device: 2^27 and more
 
 
