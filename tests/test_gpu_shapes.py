@@ -61,6 +61,12 @@ def cliques(n, k, count):
     return rng.integers(0, n // k, (count, 1)) * k + rng.integers(0, k, (count, 2))
 
 
+ONE_BLOCK = {
+    "path": (20_000, path(20_000)), "path backwards": (20_000, path(20_000)[::-1]), "short path": (4000, path(4000)),
+    "path, shuffled": (30_000, np.random.default_rng(9).permutation(path(30_000))), "lattice": (8000, lattice(80, 100)[:32_767]),
+}
+
+
 def check(n, e, mode):
     e = np.ascontiguousarray(e, dtype=np.uint32)
     d = torch.from_numpy(e.view(np.int32)).cuda()
@@ -69,6 +75,12 @@ def check(n, e, mode):
         took, usual = microseconds(lambda: g.run(d, L)), microseconds(lambda: general.run(d))
         np.testing.assert_array_equal(L.cpu().numpy().view(np.uint32), oracle.min_labels(n, e))
     assert took <= SLOWER * usual, (took, usual)
+
+
+@pytest.mark.parametrize("mode", [cc.CC_ROOT_MAXDEG, cc.CC_ROOT_IDENTITY])
+@pytest.mark.parametrize("shape", ONE_BLOCK)
+def test_one_block_run(shape, mode):
+    check(*ONE_BLOCK[shape], mode)
 
 
 VERTEX_BITS = {
