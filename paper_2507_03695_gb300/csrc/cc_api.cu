@@ -61,6 +61,7 @@ namespace {
 
 constexpr uint64_t kMaxVertices = 0x7FFFFFFFULL;
 constexpr uint64_t kHostChunk = 1ULL << 24;  // edges per cc_run_host copy chunk
+constexpr uint64_t kFullGridEdges = 1ULL << 23;  // from here the small grid fills the GPU as well
 constexpr uint64_t kZMinBytes = 128ULL << 20;  // CC_FILTER_AUTO: P at least this large gets the bitmap
 
 // Bitmap bytes for names 0 .. n (n + 1 names under R), whole 32-bit words.
@@ -734,24 +735,32 @@ cc_status cc_stream_insert(cc_graph *g, const uint32_t *edges_dev, uint64_t n_ed
   g->last = s;
   if (g->n == 0 || n_edges == 0) return CC_OK;
   const cc::EdgeSpan span = cc::split_edges(edges_dev, n_edges);
-  // Trees are taken to be settled once the handle has seen two edges per
-  // vertex: most inserted pairs then end at the filter or after one hook.
-  const bool settled = g->applied >= 2 * g->n;
+  // Trees may be settled once the handle has seen two edges per vertex: most
+  // inserted pairs then end at the filter or after one hook, on a full grid. If
+  // the list turns out to bring many vertices that nothing has joined yet (a new
+  // part of the graph), only as many blocks work as on unsettled trees; that is
+  // found on the device. R-MAT scale 16 into the empty half of a graph: 101 us with
+  // few blocks, 172 with all; 10^6 uniform pairs into R-MAT scale 20 105 and 55.
+  const bool settled = g->applied >= 2 * g->n && n_edges < kFullGridEdges && eff_filter(g);
   g->applied += n_edges;
   g->ncomp_fresh = false;
-  if (n_edges <= cc::kInsertOneBlock)
-    return from_cuda(cc::launch_insert_small(g->rf, span, g->P, (uint32_t)g->n, g->ctrl, s));
+  const uint32_t n = (uint32_t)g->n;
+  if (n_edges <= cc::kInsertOneBlock) return from_cuda(cc::launch_insert_small(g->rf, span, g->P, n, g->ctrl, s));
   CC_TRY(cudaMemsetAsync(&g->ctrl->reject, 0, sizeof(uint32_t), s));
-  CC_TRY(cc::launch_validate(span, (uint32_t)g->n, g->ctrl, s));
+  if (settled)
+    CC_TRY(cc::launch_validate_probe(g->rf, span, g->P, n, g->ctrl, s));
+  else
+    CC_TRY(cc::launch_validate(span, n, g->ctrl, s));
   uint32_t *Z = (g->z && (g->z_forced || g->z_auto_ok)) ? g->z : nullptr;
   const uint32_t *zsel = (Z && !g->z_forced) ? &g->ctrl->cert : nullptr;
-  // the last run's certificate (when its exact selection ran) picks the form;
   // a short list into settled trees takes the form for any graph, one launch
-  const bool brief = settled && !Z && n_edges < (1ULL << 20);
-  const uint32_t *hub = g->z_auto_ok && !brief ? &g->ctrl->cert : nullptr;
-  CC_TRY(cc::launch_edge_pass(g->rf, eff_filter(g), eff_ept(g), eff_block(g), span, g->P, (uint32_t)g->n, g->ctrl,
-                              &g->ctrl->reject, s, Z, zsel, false, nullptr, hub, !brief,
-                              g->z_auto_ok ? g->cert->hot : nullptr, nullptr, settled));
+  if (settled && !Z && n_edges < (1ULL << 20) && eff_ept(g) == 4 && eff_block(g) == 512)
+    return from_cuda(cc::launch_edge_pass_general(g->rf, span, g->P, n, g->ctrl, &g->ctrl->reject, s, true));
+  // the last run's certificate (when its exact selection ran) picks the form
+  const uint32_t *hub = g->z_auto_ok ? &g->ctrl->cert : nullptr;
+  CC_TRY(cc::launch_edge_pass(g->rf, eff_filter(g), eff_ept(g), eff_block(g), span, g->P, n, g->ctrl, &g->ctrl->reject,
+                              s, Z, zsel, false, nullptr, hub, true, g->z_auto_ok ? g->cert->hot : nullptr, nullptr,
+                              settled));
   return CC_OK;
 }
 

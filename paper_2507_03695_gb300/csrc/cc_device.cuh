@@ -40,7 +40,7 @@ struct RootR {
   static constexpr uint32_t kOff = 1;
   uint32_t m;
   __device__ __forceinline__ static RootR load(const Ctrl *ctrl) {
-    return RootR{*(const volatile uint32_t *)&ctrl->m};
+    return RootR{__ldca(&ctrl->m)};  // set by an earlier kernel; every warp reads it, through L1
   }
   __device__ __forceinline__ uint32_t f(uint32_t x) const { return x == m ? 0u : x + 1u; }
   __device__ __forceinline__ uint32_t finv(uint32_t c) const { return c == 0u ? m : c - 1u; }

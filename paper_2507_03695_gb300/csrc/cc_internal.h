@@ -33,7 +33,7 @@ struct alignas(128) Ctrl {
   uint32_t m;                 // planted vertex in use (written by init)
   uint32_t gmin;              // smallest vertex of m's component (min-id labels, f = R)
   uint32_t err;               // kErr* bits
-  uint32_t reject;            // the insert batch being applied failed validation
+  uint32_t reject;            // insert being applied: 1 when it failed validation (the edge pass's skip word)
   uint32_t n_cand;            // root select: candidates found by the sampled pass
   uint32_t cert;              // root select: 1 when the candidate pass proved the argmax
   uint32_t skip[3];           // chunked root select: skip words (kSkip*), set on the device
@@ -326,11 +326,12 @@ cudaError_t launch_edge_pass(bool rf, int filter, int ept, int block, const Edge
                              uint32_t *log = nullptr, const uint32_t *hub = nullptr, bool dyn = false,
                              const unsigned long long *hot = nullptr, const WideHot *wide_hot = nullptr,
                              bool settled = false);
-// The plain pass for any graph alone, its counter (ctrl->work) already zero.
+// The plain pass for any graph alone, its counter ctrl->work already zero; settled:
+// a fixed stride on a full grid, and claims where *skip lets few blocks work.
 cudaError_t launch_edge_pass_general(bool rf, const EdgeSpan &e, uint32_t *P, uint32_t n, Ctrl *ctrl,
-                                     const uint32_t *skip, cudaStream_t s);
+                                     const uint32_t *skip, cudaStream_t s, bool settled = false);
 // settled: the trees exist already, so the grid need not be kept small for the
-// edges that would all meet on the first roots.
+// edges that would all meet on the first roots (launch_validate_probe).
 // An insert of at most kInsertOneBlock pairs: validation and hooking in one
 // block.
 constexpr uint64_t kInsertOneBlock = 4096;
@@ -358,6 +359,10 @@ constexpr size_t bits_bytes(uint64_t n) { return (size_t)((n + 127) / 128 * 16);
 bool bits_pass_fits(uint64_t n_vertices, uint64_t n_edges);
 cudaError_t launch_edge_pass_bits(bool rf, const EdgeSpan &e, uint32_t *P, uint32_t n, Ctrl *ctrl, uint32_t *bits,
                                   cudaStream_t s);
+// The same for an insert of more than kInsertOneBlock pairs that may meet settled
+// trees: ctrl->reject, zero before, then tells how many blocks of the edge pass are
+// to work, and ctrl->work is zero.
+cudaError_t launch_validate_probe(bool rf, const EdgeSpan &e, const uint32_t *P, uint32_t n, Ctrl *ctrl, cudaStream_t s);
 cudaError_t launch_validate(const EdgeSpan &e, uint32_t n, Ctrl *ctrl, cudaStream_t s, uint32_t *reject = nullptr);
 cudaError_t launch_flatten(bool rf, int label_space, uint32_t *P, uint32_t n, uint32_t *L, Ctrl *ctrl,
                            cudaStream_t s);

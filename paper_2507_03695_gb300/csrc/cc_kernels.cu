@@ -134,10 +134,13 @@ __global__ void __launch_bounds__(512) k_edge_pass_direct(const uint4 *__restric
 // The hub-serving instances run only when *sel is nonzero, the other only
 // when it is zero; with sel null the launched instance runs.
 //
+// skip: nothing is done when the word is 1; k + 1: about k of the blocks work, and
+// claim (work is then given); 0: all.
 // work: the dynamic schedule. Warps claim `grab` steps of 32 * Q consecutive
 // quads at a time from *work, so warps whose edges need long searches do not
 // set the end of the kernel; null: each warp takes a fixed stride of steps.
-// The claim size is chosen by the launcher (grab_for).
+// The claim size is chosen by the launcher (grab_for). fixed: they do so only when
+// the skip word lets few blocks work.
 //
 // hot (hub instances only): the hot-vertex table of the root selection
 // (CertScratch::hot). Each block copies its vertex ids into shared memory
@@ -152,7 +155,7 @@ __global__ void __launch_bounds__(512, Q >= 4 ? (kZ ? 1 : 2) : (kZ ? 2 : (kDirec
     k_edge_pass_filtered(const uint4 *__restrict__ e4, uint64_t n_quads, const uint2 *head, const uint2 *tail,
                          uint32_t *P, uint32_t n, Ctrl *ctrl, const uint32_t *skip, uint32_t *Z,
                          const uint32_t *sel, uint32_t *log, unsigned long long *work, uint32_t grab,
-                         const unsigned long long *hot) {
+                         const unsigned long long *hot, bool fixed = false) {
   static_assert(kDirect || !kZ, "the zero-tree form resolves in place");
   // kL2 (the queue form on a parent array of at least kL2MinVertices): P is
   // read through L2 only. Its random parent loads almost never hit L1 then,
@@ -162,8 +165,16 @@ __global__ void __launch_bounds__(512, Q >= 4 ? (kZ ? 1 : 2) : (kZ ? 2 : (kDirec
   static_assert(!kL2 || (!kZ && !kDirect), "L2-only loads only in the queue form");
   constexpr bool kCG = kL2;
   extern __shared__ uint32_t ring_smem[];
-  if (skip && ld_volatile_u32(skip)) return;
-  if (sel && ((ld_volatile_u32(sel) != 0u) != (kZ || !kDirect))) return;
+  // (read through L1: every warp of the grid does)
+  bool all = true;
+  if (skip) {
+    const uint32_t w = __ldca(skip), few = w - 1u;
+    all = w == 0u || few >= gridDim.x;
+    // about that many, spread at uneven distances over the grid, so over the SMs
+    // (every eighth block of 512 ran half as fast); block 0 is one of them
+    if (!all && __umulhi(blockIdx.x * 2654435769u, gridDim.x) >= few) return;
+  }
+  if (sel && ((__ldca(sel) != 0u) != (kZ || !kDirect))) return;
   const F fn = F::load(ctrl);
   uint32_t *const S = slots<F>(P);
   const uint64_t pol = policy_evict_first();
@@ -274,7 +285,7 @@ __global__ void __launch_bounds__(512, Q >= 4 ? (kZ ? 1 : 2) : (kZ ? 2 : (kDirec
       ring.push<kCG>(S, pa != pb, fn.f(a), pa, fn.f(b), pb);
     }
   };
-  if (work) {
+  if (work && !(fixed && all)) {
     // dynamic: warps claim `grab` steps of 32 * Q consecutive quads at a time,
     // so warps whose edges need longer searches do not set the kernel's end
     const uint64_t steps = (n_quads + 32u * Q - 1) / (32u * Q);
@@ -474,11 +485,31 @@ __global__ void __launch_bounds__(kHubBlock, 1)
   }
 }
 
+// kProbe: one more block looks at kProbes pairs of quads spread over the list.
+// Where half of them join two vertices that nothing has joined yet, that part of
+// the graph still has to grow its trees, and only `few` blocks of the edge pass
+// are to work, so that fewer edges meet on the first roots. It clears the edge
+// pass's counter too. An id out of range lets no block work.
+constexpr uint32_t kProbes = 256;
+
+template <class F, bool kProbe>
 __global__ void __launch_bounds__(256) k_validate(const uint4 *__restrict__ e4, uint64_t n_quads,
                                                   const uint2 *head, const uint2 *tail, uint32_t n,
-                                                  Ctrl *ctrl, uint32_t *reject) {
+                                                  Ctrl *ctrl, uint32_t *reject, const uint32_t *P, uint32_t few) {
+  if (kProbe && blockIdx.x == gridDim.x - 1u) {
+    static_assert(kProbes == 256, "one per thread");
+    const F fn = F::load(ctrl);
+    const uint4 e = __ldg(e4 + n_quads * threadIdx.x / kProbes);
+    const bool fresh = e.x < n && e.y < n && ldP_cg(P + e.x) == fn.f(e.x) && ldP_cg(P + e.y) == fn.f(e.y);
+    const int grows = __syncthreads_count(fresh);
+    if (threadIdx.x == 0) {
+      ctrl->work = 0ULL;
+      if (2 * grows >= (int)kProbes) atomicCAS(reject, 0u, few + 1u);
+    }
+    return;
+  }
   const uint64_t pol = policy_evict_first();
-  const uint64_t T = (uint64_t)gridDim.x * blockDim.x;
+  const uint64_t T = (uint64_t)(gridDim.x - (kProbe ? 1u : 0u)) * blockDim.x;
   const uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
   bool bad = false;
   if (t == 0 && head) {
@@ -494,46 +525,40 @@ __global__ void __launch_bounds__(256) k_validate(const uint4 *__restrict__ e4, 
     bad |= (e.x >= n) | (e.y >= n) | (e.z >= n) | (e.w >= n);
   }
   if (__any_sync(0xFFFFFFFFu, bad) && (threadIdx.x & 31) == 0) {
-    atomicOr(reject, 1u);
+    atomicExch(reject, 1u);
     set_err(ctrl, kErrRange);
   }
 }
 
-// A short insert in one block, which validates all pairs, then hooks them, four
-// per thread at a time. Four launches and two memsets otherwise took longer than
-// the work.
-constexpr int kInsertBlock = 512;  // 1024 threads would not fit beside the serving executor
+// A short insert in one block, which validates all pairs, loads all parents, then
+// hooks the pairs. Four launches and two memsets otherwise took longer than the
+// work. The parents are those from before any hook: loaded later, the pairs of a
+// path in order walk down the chain that the others have built (4096 of them: 568
+// us instead of 14). They are kept in shared memory: 512 threads have no registers
+// for eight pairs each, and 1024 would not fit beside the serving executor.
+constexpr int kInsertBlock = 512;
 
 template <class F>
-__global__ void __maxnreg__(kSmallBlockRegs) k_insert_small(const uint2 *__restrict__ e, uint32_t n_edges,
-                                                            uint32_t *P, uint32_t n, Ctrl *ctrl) {
+__global__ void __maxnreg__(kSmallBlockRegs) k_insert_small(const uint2 *__restrict__ e, uint32_t n_edges, uint32_t *P,
+                                                        uint32_t n, Ctrl *ctrl) {
+  extern __shared__ uint4 pairs[];  // the ids, then the parents
   const F fn = F::load(ctrl);
   uint32_t *const S = slots<F>(P);
   bool bad = false;
-#pragma unroll 4
+#pragma unroll 2
   for (uint32_t i = threadIdx.x; i < n_edges; i += kInsertBlock) {
     const uint2 x = ld_edge(e + i);
-    bad |= x.x >= n || x.y >= n;
+    const bool ok = x.x < n && x.y < n;
+    bad |= !ok;
+    pairs[i] = make_uint4(x.x, x.y, ok ? ldP_cg(P + x.x) : 0u, ok ? ldP_cg(P + x.y) : 0u);
   }
   if (__syncthreads_or(bad)) {  // nothing is applied
     if (threadIdx.x == 0) set_err(ctrl, kErrRange);
     return;
   }
-  for (uint32_t i0 = threadIdx.x; i0 < n_edges; i0 += 4 * kInsertBlock) {
-    uint2 x[4];
-    uint32_t p[8];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint32_t i = i0 + (uint32_t)j * kInsertBlock;
-      x[j] = i < n_edges ? ld_edge(e + i) : make_uint2(0u, 0u);
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      p[2 * j] = ldP_cg(P + x[j].x);
-      p[2 * j + 1] = ldP_cg(P + x[j].y);
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) unite<true>(S, fn.f(x[j].x), p[2 * j], fn.f(x[j].y), p[2 * j + 1]);
+  for (uint32_t i = threadIdx.x; i < n_edges; i += kInsertBlock) {
+    const uint4 x = pairs[i];
+    unite<true>(S, fn.f(x.x), x.z, fn.f(x.y), x.w);
   }
 }
 
@@ -1063,28 +1088,44 @@ cudaError_t launch_edge_pass(bool rf, int filter, int ept, int block, const Edge
 
 template <class F>
 cudaError_t edge_pass_general(const EdgeSpan &e, uint32_t *P, uint32_t n, Ctrl *ctrl, const uint32_t *skip,
-                              cudaStream_t s) {
+                              cudaStream_t s, bool settled) {
   constexpr int block = 512, Q = 2;
   const size_t smem = (size_t)(block / 32) * 4 * kRing * sizeof(uint32_t);
   const void *k = (const void *)k_edge_pass_filtered<F, Q, false, true>;
-  const uint64_t per = (uint64_t)block * Q * kMinWaves;
-  const unsigned g = clamp_grid((e.n_quads + per - 1) / per, persistent_cap(k, block, smem));
+  const uint64_t per = (uint64_t)block * Q;
+  const uint64_t cap = persistent_cap(k, block, smem);
+  const unsigned few = clamp_grid((e.n_quads + per * kMinWaves - 1) / (per * kMinWaves), cap);
+  const unsigned g = settled ? clamp_grid((e.n_quads + per - 1) / per, cap) : few;
   k_edge_pass_filtered<F, Q, false, true><<<g, block, smem, s>>>(e.quads, e.n_quads, e.head, e.tail, P, n, ctrl, skip,
                                                                  nullptr, nullptr, nullptr, &ctrl->work,
-                                                                 grab_for(e.n_quads, Q, g, block), nullptr);
+                                                                 grab_for(e.n_quads, Q, few, block), nullptr, settled);
   note_launch();
   return cudaGetLastError();
 }
 
 cudaError_t launch_edge_pass_general(bool rf, const EdgeSpan &e, uint32_t *P, uint32_t n, Ctrl *ctrl,
-                                     const uint32_t *skip, cudaStream_t s) {
-  return rf ? edge_pass_general<RootR>(e, P, n, ctrl, skip, s) : edge_pass_general<RootId>(e, P, n, ctrl, skip, s);
+                                     const uint32_t *skip, cudaStream_t s, bool settled) {
+  return rf ? edge_pass_general<RootR>(e, P, n, ctrl, skip, s, settled)
+            : edge_pass_general<RootId>(e, P, n, ctrl, skip, s, settled);
 }
 
 cudaError_t launch_validate(const EdgeSpan &e, uint32_t n, Ctrl *ctrl, cudaStream_t s, uint32_t *reject) {
   if (e.n_quads == 0 && !e.head && !e.tail) return cudaSuccess;
-  const unsigned g = clamp_grid((e.n_quads + 255) / 256, persistent_cap((const void *)k_validate, 256, 0));
-  k_validate<<<g, 256, 0, s>>>(e.quads, e.n_quads, e.head, e.tail, n, ctrl, reject ? reject : &ctrl->reject);
+  const unsigned g = clamp_grid((e.n_quads + 255) / 256, persistent_cap((const void *)k_validate<RootId, false>, 256, 0));
+  k_validate<RootId, false><<<g, 256, 0, s>>>(e.quads, e.n_quads, e.head, e.tail, n, ctrl,
+                                              reject ? reject : &ctrl->reject, nullptr, 0u);
+  note_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t launch_validate_probe(bool rf, const EdgeSpan &e, const uint32_t *P, uint32_t n, Ctrl *ctrl, cudaStream_t s) {
+  const uint64_t per = 512ull * 2 * kMinWaves;  // as edge_pass_q's, for its default shape
+  const uint32_t few = clamp_grid((e.n_quads + per - 1) / per, 1u << 20);
+  const unsigned g = 1u + clamp_grid((e.n_quads + 255) / 256, persistent_cap((const void *)k_validate<RootR, true>, 256, 0));
+  if (rf)
+    k_validate<RootR, true><<<g, 256, 0, s>>>(e.quads, e.n_quads, e.head, e.tail, n, ctrl, &ctrl->reject, P, few);
+  else
+    k_validate<RootId, true><<<g, 256, 0, s>>>(e.quads, e.n_quads, e.head, e.tail, n, ctrl, &ctrl->reject, P, few);
   note_launch();
   return cudaGetLastError();
 }
@@ -1092,10 +1133,16 @@ cudaError_t launch_validate(const EdgeSpan &e, uint32_t n, Ctrl *ctrl, cudaStrea
 cudaError_t launch_insert_small(bool rf, const EdgeSpan &e, uint32_t *P, uint32_t n, Ctrl *ctrl, cudaStream_t s) {
   const uint2 *first = e.head ? e.head : (e.n_quads ? reinterpret_cast<const uint2 *>(e.quads) : e.tail);
   const uint32_t count = (uint32_t)(2 * e.n_quads + (e.head ? 1 : 0) + (e.tail ? 1 : 0));
+  static std::atomic<unsigned long long> set_r{0}, set_i{0};
+  const cudaError_t err =
+      ensure_func_attr(rf ? (const void *)k_insert_small<RootR> : (const void *)k_insert_small<RootId>,
+                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kInsertOneBlock * sizeof(uint4)), rf ? set_r : set_i);
+  if (err != cudaSuccess) return err;
+  const size_t smem = count * sizeof(uint4);
   if (rf)
-    k_insert_small<RootR><<<1, kInsertBlock, 0, s>>>(first, count, P, n, ctrl);
+    k_insert_small<RootR><<<1, kInsertBlock, smem, s>>>(first, count, P, n, ctrl);
   else
-    k_insert_small<RootId><<<1, kInsertBlock, 0, s>>>(first, count, P, n, ctrl);
+    k_insert_small<RootId><<<1, kInsertBlock, smem, s>>>(first, count, P, n, ctrl);
   note_launch();
   return cudaGetLastError();
 }
