@@ -32,6 +32,7 @@
 #include <new>
 
 #include "cc_batch.h"
+#include "cc_chunks.h"
 #include "cc_device.cuh"
 #include "cc_internal.h"
 
@@ -384,14 +385,8 @@ __device__ void filtered_phase(const BatchArgs &a, uint32_t *bits, uint32_t *rin
       // this warp's chunks that were not sampled, the next one loaded ahead
       const uint32_t full = (uint32_t)(n_e / kChunkEdges);  // chunks before a ragged last one
       const uint2 *const e_lane = a.edges + e0 + lane;
-      const uint32_t hop = nw % stride;
-      uint32_t ch = c0 + wid, phase = ch % stride;
-      auto skip = [&]() {
-        while (phase == 0u && ch < c1) {
-          ch += nw;
-          phase = hop;
-        }
-      };
+      UnsampledChunks mine(c0, stride, wid, nw);
+      uint32_t ch = mine.chunk();
       uint2 e[4];
       auto load = [&]() {
         const uint2 *const p = e_lane + (uint64_t)ch * kChunkEdges;
@@ -407,16 +402,13 @@ __device__ void filtered_phase(const BatchArgs &a, uint32_t *bits, uint32_t *rin
           }
         }
       };
-      skip();
       if (ch < c1) load();
       while (ch < c1) {
         uint2 cur[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) cur[j] = e[j];
-        ch += nw;
-        phase += hop;
-        if (phase >= stride) phase -= stride;
-        skip();
+        mine.next();
+        ch = mine.chunk();
         if (ch < c1) load();
         const uint32_t top = max(max(max(cur[0].x, cur[0].y), max(cur[1].x, cur[1].y)),
                                  max(max(cur[2].x, cur[2].y), max(cur[3].x, cur[3].y)));
