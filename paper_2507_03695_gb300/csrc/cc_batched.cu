@@ -155,13 +155,14 @@ __device__ __forceinline__ uint32_t owner_warp(const uint64_t *off, uint32_t n, 
 }
 
 // Chunks that a hooking tile holds: 3/8 of the configured tile's (the default
-// 8192 edges: 24 chunks), or fewer where that would leave less than four tiles
-// per warp. Between 15 and 30 chunks 4096 graphs take 8.4 to 8.6 ms, with 61
-// 10.2 (the last tiles leave most warps idle); 400 graphs take 1.37 ms with 6
-// and 1.69 with 2 (a warp's tiles are then of several graphs and share
-// nothing in L1); one graph of 38K edges took 0.39 ms in five tiles of 8192
-// edges and takes 0.08.
-constexpr uint64_t kTilesPerWarp = 4;
+// 8192 edges: 24 chunks), or fewer where that would leave warps without a tile.
+// Between 15 and 30 chunks 4096 graphs take 8.4 to 8.6 ms, with 61 10.2 (the last
+// tiles leave most warps idle). Smaller tiles, four per warp, spread each graph
+// over more SMs, whose warps then meet on its roots: 100 R-MAT graphs of 2^18 edges
+// 924 us, 444 like this; 200 uniform ones of 65,536 vertices with 2.5 edges each
+// 1365 and 936. One graph of 38K edges took 0.39 ms in five tiles of 8192 edges
+// and takes 0.08.
+constexpr uint64_t kTilesPerWarp = 1;
 constexpr uint32_t kTileMinChunks = 2;
 
 // Chunks of graph g that phase 1 hooks (0 when its offsets decrease).
