@@ -14,17 +14,17 @@
 //      per lane; of a graph with many edges per vertex only one chunk in
 //      sample_stride, which is enough to form its giant component;
 //   2. compression: every vertex stores its root's name, and each sampled
-//      graph gets a reference, the root that most of its vertices have;
+//      graph gets a reference, the root that most of its edges' endpoints have;
 //   3. the chunks left over, against one bit per vertex in shared memory: an
-//      edge inside the reference's tree costs two shared-memory loads;
+//      edge inside the reference's tree costs two shared-memory loads (where that
+//      tree is small, the edges are hooked as in phase 1);
 //   4. compression;
 //   5. labels: vertex tiles turn root names into graph-local ids in place.
 // Measured in ms, before (every edge hooked, one cooperative kernel) and now:
-// 4096 mixed graphs (1.18G edges) 12.2 -> 8.5, 400 graphs 2.0 -> 1.4, 40
-// graphs 0.89 -> 0.49, one graph of 38K edges 0.39 -> 0.08. Of 2000 graphs'
-// 3.8 ms phases 0 to 5 take 0.06 / 2.0 / 0.27 / 1.2 / 0.09 / 0.18: phase 1
-// waits for the dependent loads and compare-and-swaps of the searches, phase 3
-// issues 3.3 instructions per clock.
+// 4096 mixed graphs (1.18G edges) 12.2 -> 8.2, 400 graphs 2.0 -> 1.26, 40
+// graphs 0.89 -> 0.46, one graph of 38K edges 0.39 -> 0.08; lattices of 200 x 200
+// 0.62 either way. Phase 1 waits for the dependent loads and compare-and-swaps of
+// the searches, phase 3 issues 3.3 instructions per clock.
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <string.h>
@@ -32,6 +32,7 @@
 #include <new>
 
 #include "cc_batch.h"
+#include "cc_chunks.h"
 #include "cc_chunks.h"
 #include "cc_device.cuh"
 #include "cc_internal.h"
@@ -57,7 +58,7 @@ struct BatchArgs {
   uint64_t *etile_off;  // n_graphs + 1
   uint64_t *vtile_off;  // n_graphs + 1
   uint64_t *chunk_off;  // n_graphs + 1: chunks of the graphs that the filtered phase takes
-  uint32_t *ref;        // n_graphs: the root of each such graph's reference tree
+  uint32_t *ref;        // n_graphs: the root of each such graph's reference tree, and kScattered
   uint32_t tile_edges, tile_vertices;
   uint32_t hook_warps;  // warps of the hooking launch
   unsigned long long barrier_ns;  // bounded wait of every grid barrier
@@ -311,7 +312,12 @@ constexpr uint32_t kSegs = 4;
 
 // The filtered phase: the chunks of each graph that the hooking phase left,
 // against one bit per vertex in shared memory, set for the members of the
-// graph's reference tree.
+// graph's reference tree. Where that holds less than half of the graph's sampled
+// edges (kScattered in ref), the bits would let nearly every edge through, and
+// the edges are hooked as they come.
+constexpr uint32_t kMinVotes = 16;             // of 32
+constexpr uint32_t kScattered = 0x80000000u;  // names stay below 2^31
+
 __device__ void filtered_phase(const BatchArgs &a, uint32_t *bits, uint32_t *ring_words) {
   __shared__ unsigned long long s_claim;
   __shared__ uint32_t s_graph;
@@ -348,7 +354,8 @@ __device__ void filtered_phase(const BatchArgs &a, uint32_t *bits, uint32_t *rin
       t = t_end;
       const uint32_t stride = sample_stride(n_e, nv);
       const uint32_t ref = a.ref[g];
-      if (built != g) {
+      const bool scattered = (ref & kScattered) != 0u;
+      if (built != g && !scattered) {
         const uint32_t words = (nv + 31u) / 32u;
         for (uint32_t w0 = wid * 4u; w0 < words; w0 += nw * 4u) {
           uint32_t p[4];
@@ -418,6 +425,17 @@ __device__ void filtered_phase(const BatchArgs &a, uint32_t *bits, uint32_t *rin
 #pragma unroll
           for (int j = 0; j < 4; ++j)
             if (max(cur[j].x, cur[j].y) >= nv) cur[j] = make_uint2(0u, 0u);
+        }
+        if (scattered) {
+          uint32_t pa[4], pb[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            pa[j] = ldP(P + base + cur[j].x);
+            pb[j] = ldP(P + base + cur[j].y);
+          }
+#pragma unroll
+          for (int j = 0; j < 4; ++j) unite(P, base + cur[j].x, pa[j], base + cur[j].y, pb[j]);
+          continue;
         }
         uint32_t wa[4], wb[4];
 #pragma unroll
@@ -541,11 +559,14 @@ __global__ void __launch_bounds__(256) k_batch_compress(BatchArgs a) {
     for (uint64_t g = tid / 32u; g < a.n_graphs; g += T / 32u) {
       const uint64_t v0 = a.vtx_off[g], nv = a.vtx_off[g + 1] - v0;
       if (sample_stride(a.edge_off[g + 1] - a.edge_off[g], nv) == 1u) continue;
-      const uint32_t r = walk_root(P, (uint32_t)(v0 + nv * lane / 32u));
+      const uint64_t e0 = a.edge_off[g];
+      uint32_t x = a.edges[e0 + (a.edge_off[g + 1] - e0) * lane / 32u].x;  // (of edges: many vertices may have none)
+      if (x >= nv) x = 0u;
+      const uint32_t r = walk_root(P, (uint32_t)v0 + x);
       const uint32_t votes = (uint32_t)__popc(__match_any_sync(0xFFFFFFFFu, r));
-      const uint32_t best = __reduce_max_sync(0xFFFFFFFFu, votes * 32u + lane) & 31u;
-      const uint32_t ref = __shfl_sync(0xFFFFFFFFu, r, (int)best);
-      if (lane == 0) a.ref[g] = ref;
+      const uint32_t best = __reduce_max_sync(0xFFFFFFFFu, votes * 32u + lane);
+      const uint32_t ref = __shfl_sync(0xFFFFFFFFu, r, (int)(best & 31u));
+      if (lane == 0) a.ref[g] = ref | (best / 32u < kMinVotes ? kScattered : 0u);
     }
   }
   compress(P, a.vtx_off[a.n_graphs], tid, T);

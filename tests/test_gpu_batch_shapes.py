@@ -40,3 +40,17 @@ def test_a_quarter_of_the_graphs():
     # at most 0.6 of the time: it cannot fill the GPU as well, but need not be slower a graph
     parts = [(1 << 16, graphgen.rmat(16, 1 << 18, 100 + k % 20)) for k in range(400)]
     assert takes(parts[:100]) <= 0.6 * takes(parts)
+
+
+def lattice(side):
+    """Rows of a lattice with its diagonals, by first vertex."""
+    c = np.arange(side * side).reshape(side, side)
+    pairs = [(c[:, :-1], c[:, 1:]), (c[:-1], c[1:]), (c[:-1, :-1], c[1:, 1:]), (c[:-1, 1:], c[1:, :-1])]
+    e = np.concatenate([np.stack([a.ravel(), b.ravel()], 1) for a, b in pairs])
+    return e[np.argsort(e[:, 0], kind="stable")]
+
+
+def test_lattices():
+    # with 40% more vertices, of no edges, the same graphs are hooked whole: the sampled route may cost a third more
+    e = lattice(200)
+    assert takes([(40_000, e)] * 200) <= 1.33 * takes([(56_000, e)] * 200)
