@@ -932,9 +932,9 @@ def bench_csr(args, cc, graphs, torch, stream):
 
 
 def bench_batched(args, cc, graphgen, torch, stream):
-    """The mixed batch of many small graphs: one tuned, CUDA-graph-captured
-    persistent launch (cc_run_batched) against the plain path of one cc_run
-    per graph (f = id, handles created beforehand)."""
+    """The mixed batch of many small graphs: one tuned call (cc_run_batched),
+    captured in a CUDA graph, against the plain path of one cc_run per graph
+    (f = id, handles created beforehand)."""
     import numpy as np
     d = graphgen.batch_dev(args.batched_graphs, graphgen.BATCH_SEED)
     torch.cuda.synchronize()

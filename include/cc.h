@@ -134,7 +134,8 @@ typedef struct cc_options {
   int32_t block_size;        /* edge-pass threads per block (128, 256, 512); 0 = 512 */
   int32_t edges_per_thread;  /* edges per thread per iteration (2, 4 or 8); 0 = auto */
   int32_t sample_stride;     /* sampled root select keeps 1 group in k; 0 = 16     */
-  int32_t timing;            /* nonzero: record per-phase times (cc_phase_times)  */
+  int32_t timing;            /* nonzero: record per-phase times (cc_phase_times); small graphs
+                                then run phase by phase, not in one launch        */
   uint64_t hbm_budget_bytes; /* device bytes the handle may own; 0 = free memory  */
   int32_t initial_push;      /* cc_initial_push, default CC_PUSH_AUTO              */
   int32_t reserved32;        /* must be zero                                       */

@@ -264,8 +264,9 @@ constexpr uint32_t kNeverDirect = 33;
 // because name 0 is never hooked; a stale 0 bit only costs the parent load
 // it would have saved. Name 0 itself (the tree's root m) never gets its bit:
 // the many hooks onto m would all send an atomic to the one word that holds
-// it. A lookup of m then loads P of m, which is 0 (the hot-vertex table
-// answers for m first where there is one).
+// it. A lookup of m then loads P of m, which is 0 (the hot-vertex tables learn
+// from the bitmap where there is one, and so never know m; without the bitmap
+// they learn m like any other vertex).
 __device__ __forceinline__ bool zbit(const uint32_t *Z, uint32_t c) {
   uint32_t w;
   asm volatile("ld.global.u32 %0, [%1];" : "=r"(w) : "l"(Z + (c >> 5)) : "memory");
