@@ -745,7 +745,11 @@ cc_status cc_stream_insert(cc_graph *g, const uint32_t *edges_dev, uint64_t n_ed
   g->applied += n_edges;
   g->ncomp_fresh = false;
   const uint32_t n = (uint32_t)g->n;
-  if (n_edges <= cc::kInsertOneBlock) return from_cuda(cc::launch_insert_small(g->rf, span, g->P, n, g->ctrl, s));
+  if (n_edges <= cc::kInsertOneBlock) {
+    const cc::ExecutorBlocks executor(g->device);
+    return from_cuda(cc::launch_insert_small(g->rf, span, g->P, n, g->ctrl, s,
+                                             executor.count() <= (uint32_t)cc::kExecutorDefault));
+  }
   CC_TRY(cudaMemsetAsync(&g->ctrl->reject, 0, sizeof(uint32_t), s));
   if (settled)
     CC_TRY(cc::launch_validate_probe(g->rf, span, g->P, n, g->ctrl, s));

@@ -105,6 +105,7 @@ class ExecutorBlocks {
 };
 void executor_announce(int device, uint32_t blocks_per_sm);
 void executor_withdraw(int device, uint32_t blocks_per_sm);
+cudaError_t load_kernels_beside_executor();
 
 // Sets a kernel attribute once per device. Setting a function attribute can
 // make the host wait for the device, so it is done on first use only, never
@@ -335,7 +336,8 @@ cudaError_t launch_edge_pass_general(bool rf, const EdgeSpan &e, uint32_t *P, ui
 // An insert of at most kInsertOneBlock pairs: validation and hooking in one
 // block.
 constexpr uint64_t kInsertOneBlock = 4096;
-cudaError_t launch_insert_small(bool rf, const EdgeSpan &e, uint32_t *P, uint32_t n, Ctrl *ctrl, cudaStream_t s);
+cudaError_t launch_insert_small(bool rf, const EdgeSpan &e, uint32_t *P, uint32_t n, Ctrl *ctrl, cudaStream_t s,
+                                bool large_block);
 // dyn: warps claim their edges from a counter in ctrl (reset on s before the
 // launch), so at most one dynamic edge pass per Ctrl may be in flight.
 // Sets *reject (ctrl->reject when null) and the range error bit when an id is >= n.

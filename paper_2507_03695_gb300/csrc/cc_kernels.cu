@@ -534,12 +534,14 @@ __global__ void __launch_bounds__(256) k_validate(const uint4 *__restrict__ e4, 
 // hooks the pairs. Four launches and two memsets otherwise took longer than the
 // work. The parents are those from before any hook: loaded later, the pairs of a
 // path in order walk down the chain that the others have built (4096 of them: 568
-// us instead of 14). They are kept in shared memory: 512 threads have no registers
-// for eight pairs each, and 1024 would not fit beside the serving executor.
-constexpr int kInsertBlock = 512;
+// us instead of 14). They are kept in shared memory: the registers that are left
+// beside the serving executor do not hold them. 1024 threads fit beside three of
+// its blocks per SM, 512 beside four.
+template <int kInsertBlock>
+constexpr int kInsertRegs = kInsertBlock == 1024 ? kBesideExecutorRegs / 1024 / 8 * 8 : kSmallBlockRegs;
 
-template <class F>
-__global__ void __maxnreg__(kSmallBlockRegs) k_insert_small(const uint2 *__restrict__ e, uint32_t n_edges, uint32_t *P,
+template <class F, int kInsertBlock>
+__global__ void __maxnreg__(kInsertRegs<kInsertBlock>) k_insert_small(const uint2 *__restrict__ e, uint32_t n_edges, uint32_t *P,
                                                         uint32_t n, Ctrl *ctrl) {
   extern __shared__ uint4 pairs[];  // the ids, then the parents
   const F fn = F::load(ctrl);
@@ -1130,21 +1132,48 @@ cudaError_t launch_validate_probe(bool rf, const EdgeSpan &e, const uint32_t *P,
   return cudaGetLastError();
 }
 
-cudaError_t launch_insert_small(bool rf, const EdgeSpan &e, uint32_t *P, uint32_t n, Ctrl *ctrl, cudaStream_t s) {
-  const uint2 *first = e.head ? e.head : (e.n_quads ? reinterpret_cast<const uint2 *>(e.quads) : e.tail);
-  const uint32_t count = (uint32_t)(2 * e.n_quads + (e.head ? 1 : 0) + (e.tail ? 1 : 0));
-  static std::atomic<unsigned long long> set_r{0}, set_i{0};
+namespace {
+template <class F, int kBlock>
+cudaError_t insert_small(const uint2 *first, uint32_t count, uint32_t *P, uint32_t n, Ctrl *ctrl, cudaStream_t s) {
+  static_assert(beside_executor(kBlock, kInsertRegs<kBlock>), "inserts run beside a busy server");
+  static std::atomic<unsigned long long> smem_set{0};
   const cudaError_t err =
-      ensure_func_attr(rf ? (const void *)k_insert_small<RootR> : (const void *)k_insert_small<RootId>,
-                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kInsertOneBlock * sizeof(uint4)), rf ? set_r : set_i);
+      ensure_func_attr((const void *)k_insert_small<F, kBlock>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)(kInsertOneBlock * sizeof(uint4)), smem_set);
   if (err != cudaSuccess) return err;
-  const size_t smem = count * sizeof(uint4);
-  if (rf)
-    k_insert_small<RootR><<<1, kInsertBlock, smem, s>>>(first, count, P, n, ctrl);
-  else
-    k_insert_small<RootId><<<1, kInsertBlock, smem, s>>>(first, count, P, n, ctrl);
+  k_insert_small<F, kBlock><<<1, kBlock, count * sizeof(uint4), s>>>(first, count, P, n, ctrl);
   note_launch();
   return cudaGetLastError();
+}
+}  // namespace
+
+cudaError_t launch_insert_small(bool rf, const EdgeSpan &e, uint32_t *P, uint32_t n, Ctrl *ctrl, cudaStream_t s,
+                                bool large_block) {
+  const uint2 *first = e.head ? e.head : (e.n_quads ? reinterpret_cast<const uint2 *>(e.quads) : e.tail);
+  const uint32_t count = (uint32_t)(2 * e.n_quads + (e.head ? 1 : 0) + (e.tail ? 1 : 0));
+  if (large_block)
+    return rf ? insert_small<RootR, 1024>(first, count, P, n, ctrl, s) : insert_small<RootId, 1024>(first, count, P, n, ctrl, s);
+  return rf ? insert_small<RootR, 512>(first, count, P, n, ctrl, s) : insert_small<RootId, 512>(first, count, P, n, ctrl, s);
+}
+
+// The kernels that single-graph calls take only while a server is open. With lazy
+// module loading a first launch may wait for the device to be idle, which beside an
+// executor it is not; asking for the attributes loads them.
+cudaError_t load_kernels_beside_executor() {
+  const void *const kernels[] = {
+      (const void *)k_edge_pass_filtered<RootR, 2, false, false, false>,
+      (const void *)k_edge_pass_filtered<RootR, 2, false, false, true>,
+      (const void *)k_edge_pass_filtered<RootR, 2, false, true>,
+      (const void *)k_edge_pass_filtered<RootId, 2, false, true>,
+      (const void *)k_insert_small<RootR, 512>,
+      (const void *)k_insert_small<RootId, 512>,
+  };
+  for (const void *k : kernels) {
+    cudaFuncAttributes a;
+    const cudaError_t e = cudaFuncGetAttributes(&a, k);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t launch_gmin_probe(uint32_t *P, uint32_t n, Ctrl *ctrl, cudaStream_t s) {

@@ -1363,6 +1363,7 @@ cc_status cc_server_create(const cc_server_config *cfg_in, cc_server **out) {
     s->announced = true;
     e = cudaDeviceSynchronize();  // what was enqueued before may need whole SMs
   }
+  if (e == cudaSuccess) e = cc::load_kernels_beside_executor();
   if (e == cudaSuccess) e = cudaMalloc((void **)&s->arena_base, cfg.hbm_budget_bytes);
   if (e == cudaSuccess) e = cudaHostAlloc((void **)&s->hs, sizeof(HostShared), cudaHostAllocMapped);
   if (e == cudaSuccess) e = cudaHostGetDevicePointer((void **)&s->hs_dev, s->hs, 0);

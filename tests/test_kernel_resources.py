@@ -17,7 +17,7 @@ LISTED = {
     "k_select_begin": (256, 0), "k_degree_sampled": (256, 0), "k_degree_certify": (512, 32 << 10),
     "k_select_candidates": (512, 0), "k_argmax_u32": (256, 0), "k_degree": (256, 0), "k_wide_hot_pack": (256, 0),
     "k_init": (256, 0), "k_tiny": (1024, 4 * (48 << 10)), "k_bits_link": (256, 0), "k_bits_build": (256, 0),
-    "k_bits_filter": (640, (1504 << 10) // 8 + 20 * 2 * 64 * 4), "k_insert_small": (512, 0), "k_validate": (256, 0),
+    "k_bits_filter": (640, (1504 << 10) // 8 + 20 * 2 * 64 * 4), "k_insert_small": (512, 64 << 10), "k_validate": (256, 0),
     "k_gmin_probe": (256, 0), "k_flatten4": (256, 0), "k_flatten": (256, 0), "k_connected": (256, 0),
     "k_count_roots": (256, 0), "k_csr_maxlen": (256, 0), "k_csr_tile_rows": (256, 0), "k_edge_pass_csr": (256, 0),
 }
