@@ -51,9 +51,11 @@ constexpr uint32_t kChunkQuads = 64;  // 128 edges, four per lane of a warp
 constexpr int kFilterBlock = 640, kFilterRegs = 40;
 static_assert(beside_executor(kFilterBlock, kFilterRegs), "the filter runs beside a busy server");
 constexpr int kLinkBlock = 256;
-constexpr size_t kFilterQueueBytes = (kFilterBlock / 32) * 2 * kRing * sizeof(uint32_t);
-static_assert(kBitsVertices / 8 + kFilterQueueBytes <= kBesideExecutorSmem, "the bits and the queues fit beside the executor");
-// Two blocks on an SM where their bits fit.
+constexpr size_t filter_queue_bytes(int block) { return (size_t)(block / 32) * 2 * kRing * sizeof(uint32_t); }
+static_assert(kBitsVertices / 8 + filter_queue_bytes(kFilterBlock) <= kBesideExecutorSmem, "the bits and the queues fit beside the executor");
+// Two blocks on an SM where their bits fit, then of 512 threads: R-MAT scale 18 (f =
+// id) 119 us with two of 640, 111 with these.
+constexpr int kFilterPairBlock = 512;
 constexpr size_t kFilterPairBytes = kSmemPerSM / 2 - kSmemPerBlock;
 
 // Linking rounds and their samples: two edges per vertex in the first round, a
@@ -80,6 +82,12 @@ struct Rounds {
 // than the atomics (uniform graph of 1.5M vertices: 28 -> 75 us), only those whose
 // target is often met by the block's first edges: 2^21 edges of a star whose
 // centre has the largest id took 2548 us with an atomic each.
+__device__ __forceinline__ uint4 ld_quad_now(const uint4 *a) {  // kept where it stands in the program
+  uint4 v;
+  asm volatile("ld.global.nc.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(a));
+  return v;
+}
+
 constexpr uint32_t kCentreBits = 8, kCentreCount = kLinkBlock / 32;
 __device__ __forceinline__ uint32_t centre_slot(uint32_t x) { return (x * 2654435761u) >> (32u - kCentreBits); }
 
@@ -88,9 +96,26 @@ __global__ void __launch_bounds__(kLinkBlock) k_bits_link(const uint4 *__restric
                                                           uint32_t r, uint32_t *P, uint32_t n, Ctrl *ctrl) {
   __shared__ uint32_t centre[1u << kCentreBits];
   const F fn = F::load(ctrl);
-  uint32_t linked = 0;  // rounds that have linked
-  bool flat = true;
+  uint32_t *const S = slots<F>(P);
+  const uint32_t lane = threadIdx.x & 31u;
+  uint64_t step, q0;
+  uint4 e[2];
+  auto start = [&](uint32_t stride) {  // other edges than the round before
+    step = (uint64_t)stride * kChunkQuads;
+    q0 = ((uint64_t)blockIdx.x * (kLinkBlock / 32) + (threadIdx.x >> 5)) * step + r % stride * kChunkQuads;
+  };
+  auto load = [&]() {
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const uint64_t q = q0 + 32u * j + lane;
+      e[j] = q < n_quads ? ld_quad_now(e4 + q) : make_uint4(0u, 0u, 0u, 0u);
+    }
+  };
+  start(rounds.chunk_stride[r]);
+  load();  // while it is found whether the rounds before have all linked
   if (!kFirst) {
+    uint32_t linked = 0;  // rounds that have linked
+    bool flat = true;
     uint32_t deep[kRounds];  // through L1: every warp reads them
 #pragma unroll
     for (uint32_t j = 0; j < kRounds; ++j) deep[j] = ldP(&ctrl->deep[j]);
@@ -100,33 +125,31 @@ __global__ void __launch_bounds__(kLinkBlock) k_bits_link(const uint4 *__restric
       linked += flat ? 1u : 0u;
       flat = deep[j] == 0u;
     }
-  }
-  if (blockIdx.x == 0 && threadIdx.x == 0) ctrl->deep[r] = 0u;
-  if (!flat) return;
-  const uint32_t stride = rounds.chunk_stride[linked], first = r % stride;  // other edges than the round before
-  uint32_t *const S = slots<F>(P);
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint64_t step = (uint64_t)stride * kChunkQuads;
-  const uint64_t hop = (uint64_t)gridDim.x * (kLinkBlock / 32) * step;
-  if (kFirst) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctrl->deep[r] = 0u;
+    if (!flat) return;
+    if (linked != r) {
+      start(rounds.chunk_stride[linked]);
+      load();
+    }
+  } else {
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctrl->deep[r] = 0u;
     for (uint32_t i = threadIdx.x; i < 1u << kCentreBits; i += kLinkBlock) centre[i] = 0u;
     __syncthreads();
   }
+  const uint64_t hop = (uint64_t)gridDim.x * (kLinkBlock / 32) * step;
   bool counted = !kFirst;
-  for (uint64_t q0 = ((uint64_t)blockIdx.x * (kLinkBlock / 32) + (threadIdx.x >> 5)) * step + first * kChunkQuads;
-       q0 < n_quads || !counted; q0 += hop) {
+  while (q0 < n_quads || !counted) {
     uint32_t x[8], p[8];
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-      const uint64_t q = q0 + 32u * j + lane;
-      uint4 e = make_uint4(0u, 0u, 0u, 0u);
-      if (q < n_quads) e = __ldg(e4 + q);
-      if (max(max(e.x, e.y), max(e.z, e.w)) >= n) e = make_uint4(0u, 0u, 0u, 0u);  // reported by the filter
-      x[4 * j] = e.x;
-      x[4 * j + 1] = e.y;
-      x[4 * j + 2] = e.z;
-      x[4 * j + 3] = e.w;
+      if (max(max(e[j].x, e[j].y), max(e[j].z, e[j].w)) >= n) e[j] = make_uint4(0u, 0u, 0u, 0u);  // reported by the filter
+      x[4 * j] = e[j].x;
+      x[4 * j + 1] = e[j].y;
+      x[4 * j + 2] = e[j].z;
+      x[4 * j + 3] = e[j].w;
     }
+    q0 += hop;
+    load();
 #pragma unroll
     for (int i = 0; i < 8; ++i) p[i] = kFirst ? fn.f(x[i]) : ldP(P + x[i]);
     if (!counted) {  // once per block, by every thread
@@ -238,8 +261,8 @@ __global__ void __launch_bounds__(256) k_bits_build(const uint4 *__restrict__ e4
   if (threadIdx.x == 0 && s_deep) ctrl->deep[r] = 1u;
 }
 
-// Step 3. Blocks of 20 warps, because one of 32 would not fit beside the serving
-// executor's; a warp's next chunk is loaded while it works on one. Long lists are
+// Step 3. One block of 20 warps on an SM, or two of 16, because one of 32 would not
+// fit beside the serving executor's; a warp's next chunk is loaded while it works on one. Long lists are
 // claimed kGrab chunks at a time: with a fixed split into one block per SM the
 // pass took either 235 or 550 us on R-MAT scale 20 with 2^26 edges, from run to
 // run. Whole calls with one static block of 32 warps, 16 warps and like this, us:
@@ -257,14 +280,14 @@ __global__ void __maxnreg__(kFilterRegs)
   const uint32_t ref = ldP(&ctrl->ref);
   const uint32_t groups = (n + 127u) / 128u;
   uint32_t *const bits = smem;
-  for (uint32_t i = threadIdx.x; i < groups; i += kFilterBlock)
+  for (uint32_t i = threadIdx.x; i < groups; i += blockDim.x)
     reinterpret_cast<uint4 *>(bits)[i] = __ldg(reinterpret_cast<const uint4 *>(all_bits) + i);
   const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5, lt_mask = (1u << lane) - 1u;
   // a queue of ids per warp (top bit: marked), as deep as the warp ring's
   uint32_t *const qa = smem + 4u * groups + wid * 2 * kRing, *const qb = qa + kRing;
   uint32_t q_head = 0, q_tail = 0;
   __syncthreads();
-  const uint64_t t = blockIdx.x * (uint64_t)kFilterBlock + threadIdx.x;
+  const uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
   if (t == 0 && head) single_edge<F, true>(P, fn, head, n, ctrl);
   if (t == 1 && tail) single_edge<F, true>(P, fn, tail, n, ctrl);
   auto resolve = [&](uint32_t count) {
@@ -317,7 +340,7 @@ __global__ void __maxnreg__(kFilterRegs)
       if (grab > 1u) {
         claim();
       } else {
-        ch += gridDim.x * (kFilterBlock / 32) - 1u;
+        ch += gridDim.x * (blockDim.x / 32u) - 1u;
         end = ch + 1u;
       }
     }
@@ -383,13 +406,14 @@ cudaError_t bits_pass(const EdgeSpan &e, uint32_t *P, uint32_t n, Ctrl *ctrl, ui
   const void *k = (const void *)k_bits_filter<F>;
   static std::atomic<unsigned long long> smem_set{0};
   const cudaError_t err = ensure_func_attr(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)(kBitsVertices / 8 + kFilterQueueBytes), smem_set);
+                                           (int)(kBitsVertices / 8 + filter_queue_bytes(kFilterBlock)), smem_set);
   if (err != cudaSuccess) return err;
-  const size_t smem = bits_bytes(n) + kFilterQueueBytes;
-  const unsigned gf = clamp_grid((chunks + kFilterBlock / 32 - 1) / (kFilterBlock / 32),
-                                 (uint64_t)num_sms() * (smem <= kFilterPairBytes ? 2u : 1u));
-  const uint32_t grab = chunks >= (uint64_t)gf * (kFilterBlock / 32) * 4u * kGrab ? kGrab : 1u;
-  k_bits_filter<F><<<gf, kFilterBlock, smem, s>>>(e.quads, e.n_quads, e.head, e.tail, P, n, ctrl, bits, grab);
+  const bool pair = bits_bytes(n) + filter_queue_bytes(kFilterPairBlock) <= kFilterPairBytes;
+  const unsigned block = pair ? kFilterPairBlock : kFilterBlock, warps = block / 32;
+  const size_t smem = bits_bytes(n) + filter_queue_bytes(block);
+  const unsigned gf = clamp_grid((chunks + warps - 1) / warps, (uint64_t)num_sms() * (pair ? 2u : 1u));
+  const uint32_t grab = chunks >= (uint64_t)gf * warps * 4u * kGrab ? kGrab : 1u;
+  k_bits_filter<F><<<gf, block, smem, s>>>(e.quads, e.n_quads, e.head, e.tail, P, n, ctrl, bits, grab);
   note_launch();
   // step 4, or nothing (the counter was reset with step 3's)
   return launch_edge_pass_general(F::kRF, e, P, n, ctrl, &ctrl->marked, s);
