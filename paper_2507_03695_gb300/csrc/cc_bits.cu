@@ -30,8 +30,8 @@
 //      (many components of one size, meshes that the rounds joined in part), the
 //      filter would queue nearly every edge: the general pass takes its place.
 //      The choice is made on the device.
-// Whole calls under f = id, us, general pass and this one: R-MAT scale 16 88 -> 72,
-// 18 182 -> 92, 20 with 2^26 edges 1200 -> 300; uniform, 1.5M vertices with three
+// Whole calls under f = id, us, general pass and this one: R-MAT scale 16 88 -> 74,
+// 18 178 -> 92, 20 with 2^26 edges 1200 -> 308; uniform, 1.5M vertices with three
 // edges each 350 -> 158; lattice of 1000 x 1000 with eight neighbours 198 -> 100, of
 // 100^3 with 26 182 -> 200; star whose centre has the largest id 370 -> 198; cliques
 // of ten 196 -> 222. What bounds it: at scale 16 the launches (eleven of 2 to 4 us,
@@ -262,13 +262,13 @@ __global__ void __launch_bounds__(256) k_bits_build(const uint4 *__restrict__ e4
 }
 
 // Step 3. One block of 20 warps on an SM, or two of 16, because one of 32 would not
-// fit beside the serving executor's; a warp's next chunk is loaded while it works on one. Long lists are
-// claimed kGrab chunks at a time: with a fixed split into one block per SM the
-// pass took either 235 or 550 us on R-MAT scale 20 with 2^26 edges, from run to
-// run. Whole calls with one static block of 32 warps, 16 warps and like this, us:
-// R-MAT scale 18 (f = id) 111 / 106 / 109, 19 207 / 195 / 196, 20 with 2^26 edges
-// 539 / 513 / 481, 1,000,003 vertices with 16M edges 270 / 288 / 279; 28 warps of
-// 32 registers, with spills, 116 / 197 / 466 / 270.
+// fit beside the serving executor's; a warp's next chunk is loaded while it works on
+// one. Long lists are claimed kGrab chunks at a time: with a fixed split into one
+// block per SM the pass took either 235 or 550 us on R-MAT scale 20 with 2^26 edges,
+// from run to run. Whole calls with one block of 32 warps and a fixed split, and like
+// this, us: R-MAT scale 18 (f = id) 111 and 106, 19 206 and 192, 20 with 2^26 edges 538
+// and 480, 1,000,003 vertices with 16M edges 270 and 260; with one block of 28 warps of
+// 32 registers, which spill, 116 / 197 / 466 / 270.
 template <class F>
 __global__ void __maxnreg__(kFilterRegs)
     k_bits_filter(const uint4 *__restrict__ e4, uint64_t n_quads, const uint2 *head, const uint2 *tail, uint32_t *P,
