@@ -103,7 +103,7 @@ class ExecutorBlocks {
  private:
   uint32_t n_;
 };
-void executor_announce(int device, uint32_t blocks_per_sm);
+uint32_t executor_announce(int device, uint32_t blocks_per_sm);  // returns the count before
 void executor_withdraw(int device, uint32_t blocks_per_sm);
 cudaError_t load_kernels_beside_executor();
 

@@ -860,6 +860,14 @@ namespace {
 struct Servers {
   std::shared_mutex mu;
   std::map<int, std::array<uint32_t, 9>> open;  // per device, servers by executor blocks per SM
+  uint32_t most(int device) const {
+    uint32_t n = 0;
+    const auto it = open.find(device);
+    if (it != open.end())
+      for (uint32_t k = 1; k < it->second.size(); ++k)
+        if (it->second[k]) n = k;
+    return n;
+  }
 };
 Servers &servers() {
   static Servers *s = new Servers();  // outlives every server
@@ -867,20 +875,18 @@ Servers &servers() {
 }
 }  // namespace
 
-ExecutorBlocks::ExecutorBlocks(int device) : n_(0) {
-  Servers &s = servers();
-  s.mu.lock_shared();
-  const auto it = s.open.find(device);
-  if (it != s.open.end())
-    for (uint32_t k = 1; k < it->second.size(); ++k)
-      if (it->second[k]) n_ = k;
+ExecutorBlocks::ExecutorBlocks(int device) {
+  servers().mu.lock_shared();
+  n_ = servers().most(device);
 }
 ExecutorBlocks::~ExecutorBlocks() { servers().mu.unlock_shared(); }
 
-void executor_announce(int device, uint32_t blocks_per_sm) {
+uint32_t executor_announce(int device, uint32_t blocks_per_sm) {
   Servers &s = servers();
   std::lock_guard<std::shared_mutex> lk(s.mu);
+  const uint32_t before = s.most(device);
   s.open[device][blocks_per_sm < 8 ? blocks_per_sm : 8]++;
+  return before;
 }
 void executor_withdraw(int device, uint32_t blocks_per_sm) {
   Servers &s = servers();

@@ -1359,9 +1359,10 @@ cc_status cc_server_create(const cc_server_config *cfg_in, cc_server **out) {
   s->hold_left = cfg.fault_hold_publish_us ? 1u : 0u;
   cudaError_t e = cudaGetDevice(&s->device);
   if (e == cudaSuccess) {
-    cc::executor_announce(s->device, cfg.executor_blocks_per_sm);
+    const uint32_t before = cc::executor_announce(s->device, cfg.executor_blocks_per_sm), kept = cc::kExecutorDefault;
     s->announced = true;
-    e = cudaDeviceSynchronize();  // what was enqueued before may need whole SMs
+    // what was enqueued before may need more of the SMs than this executor leaves
+    if (before == 0 || (before <= kept && cfg.executor_blocks_per_sm > kept)) e = cudaDeviceSynchronize();
   }
   if (e == cudaSuccess) e = cc::load_kernels_beside_executor();
   if (e == cudaSuccess) e = cudaMalloc((void **)&s->arena_base, cfg.hbm_budget_bytes);
